@@ -34,36 +34,114 @@ struct CompPtrs {
   const float *f[6];
 };
 
-// one thread per cell, x fastest; record = 12 float4 with the components
-// interleaved in pairs (Ex, Ey), (Ez, Bx), (By, Bz): float 16 p + 2 k + h is
-// coefficient a_k of component 2 p + h
-__global__ void pack_cells_kernel(const __grid_constant__ CompPtrs src, int nx, int ny, int nz,
-                                  float4 *__restrict__ out) {
-  const long long cx = nx - 1, cy = ny - 1;
-  const long long cells = cx * cy * (long long)(nz - 1);
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long sy = nx, sz = (long long)nx * ny;
-  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < cells; c += stride) {
-    const long long iz = c / (cx * cy);
-    const long long r = c - iz * cx * cy;
-    const long long iy = r / cx;
-    const long long ix = r - iy * cx;
-    const long long b = iz * sz + iy * sy + ix;
-    float *rec = reinterpret_cast<float *>(out + 12 * c);
-    for (int comp = 0; comp < 6; ++comp) {
-      const float *f = src.f[comp];
-      const double c000 = f[b], c100 = f[b + 1], c010 = f[b + sy], c110 = f[b + sy + 1];
-      const double c001 = f[b + sz], c101 = f[b + sz + 1], c011 = f[b + sz + sy],
-                   c111 = f[b + sz + sy + 1];
-      const double a1 = c100 - c000, a2 = c010 - c000, a3 = c001 - c000;
-      const double a4 = (c110 - c100) - (c010 - c000);
-      const double a5 = (c011 - c010) - (c001 - c000);
-      const double a6 = (c101 - c100) - (c001 - c000);
-      const double a7 = ((c111 - c110) - (c101 - c100)) - ((c011 - c010) - (c001 - c000));
-      const double a[8] = {c000, a1, a2, a3, a4, a5, a6, a7};
-      float *r = rec + 16 * (comp >> 1) + (comp & 1);
-      for (int k = 0; k < 8; ++k) r[2 * k] = (float)a[k];
+// x - y as hi + lo exactly (Knuth's TwoSum of x and -y)
+struct Diff {
+  float hi, lo;
+};
+__device__ __forceinline__ Diff two_diff(float x, float y) {
+  const float s = __fsub_rn(x, y);
+  const float b = __fsub_rn(s, x);
+  return {s, __fsub_rn(__fsub_rn(x, __fsub_rn(s, b)), __fadd_rn(y, b))};
+}
+// (p - q) as a float-float sum, and rounded to one float
+__device__ __forceinline__ Diff diff(Diff p, Diff q) {
+  Diff d = two_diff(p.hi, q.hi);
+  d.lo = __fadd_rn(d.lo, __fsub_rn(p.lo, q.lo));
+  return d;
+}
+__device__ __forceinline__ float diff_rn(Diff p, Diff q) {
+  const Diff d = diff(p, q);
+  return __fadd_rn(d.hi, d.lo);
+}
+
+// The eight coefficients of one component from its corners c[i + 2 j + 4 k].
+// The differences of differences are formed in float-float arithmetic: the
+// first differences exactly, the second and third to ~2^-48 relative, so a
+// coefficient is the correctly rounded one but where the exact value lies
+// within ~2^-48 of a rounding boundary.  In double each difference would run
+// on the FP64 pipe, which together with the conversions is what bounded the
+// whole copy (see pack_cells_kernel).  A corner that is not finite, or one so
+// large that a float difference overflows, shows up in a5, a6 or a7 (between
+// them they take in every difference): then the coefficients come from the
+// plain double differences.
+__device__ __forceinline__ void cell_coeffs(const float c[8], float a[8]) {
+  const Diff x00 = two_diff(c[1], c[0]), x10 = two_diff(c[3], c[2]);
+  const Diff x01 = two_diff(c[5], c[4]), x11 = two_diff(c[7], c[6]);
+  const Diff y0 = two_diff(c[2], c[0]), y1 = two_diff(c[6], c[4]);
+  a[0] = c[0];
+  a[1] = x00.hi;
+  a[2] = y0.hi;
+  a[3] = __fsub_rn(c[4], c[0]);
+  const Diff xy0 = diff(x10, x00), xy1 = diff(x11, x01);
+  a[4] = __fadd_rn(xy0.hi, xy0.lo);
+  a[5] = diff_rn(y1, y0);
+  a[6] = diff_rn(x01, x00);
+  a[7] = diff_rn(xy1, xy0);
+  if (!(fabsf(a[5]) + fabsf(a[6]) + fabsf(a[7]) <= 3.402823466e38f)) {
+    double d[8];
+    for (int k = 0; k < 8; ++k) d[k] = (double)c[k];
+    a[1] = (float)(d[1] - d[0]);
+    a[2] = (float)(d[2] - d[0]);
+    a[3] = (float)(d[4] - d[0]);
+    a[4] = (float)((d[3] - d[1]) - (d[2] - d[0]));
+    a[5] = (float)((d[6] - d[2]) - (d[4] - d[0]));
+    a[6] = (float)((d[5] - d[1]) - (d[4] - d[0]));
+    a[7] = (float)(((d[7] - d[3]) - (d[5] - d[1])) - ((d[6] - d[2]) - (d[4] - d[0])));
+  }
+}
+
+// Record = 12 float4 with the components interleaved in pairs (Ex, Ey),
+// (Ez, Bx), (By, Bz): float 16 p + 2 k + h is coefficient a_k of component
+// 2 p + h.  Bound by the writes: 192 bytes per cell against 24 read.  A warp
+// takes 32 consecutive cells, lane l computing cell l, and turns its 6 KB of
+// records around in shared memory (slot k of cell l at [k][l], one float4 of
+// padding per row, so both directions are free of bank conflicts up to the
+// wrap from one record to the next), so that every store is 512 contiguous
+// bytes.  Measured at 256^3 (3.59 GB): 6.88 ms with
+// double differences and 4-byte stores 8 bytes apart, 0.69 ms so (5.19 TB/s).
+constexpr int kPackWarps = 8;
+constexpr int kPackRow = 33;  // float4 per slot row
+
+__global__ void __launch_bounds__(32 * kPackWarps)
+    pack_cells_kernel(const __grid_constant__ CompPtrs src, int nx, int ny, int nz, float4 *__restrict__ out) {
+  extern __shared__ __align__(16) float4 s_rec[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float4 *rec = s_rec + warp * (12 * kPackRow);
+  const unsigned cx = nx - 1, cy = ny - 1;
+  const unsigned cells = cx * cy * (unsigned)(nz - 1);  // fewer than the nodes, so below 2^31
+  const int sy = nx, sz = nx * ny;
+  const unsigned n_warps = gridDim.x * kPackWarps;
+  const unsigned groups = (cells + 31u) / 32u;
+  for (unsigned g = blockIdx.x * kPackWarps + warp; g < groups; g += n_warps) {
+    const unsigned first = 32u * g;
+    const unsigned n = cells - first < 32u ? cells - first : 32u;
+    const unsigned c = first + (lane < (int)n ? lane : (int)n - 1);  // spare lanes repeat the last cell
+    const unsigned iz = c / (cx * cy);
+    const unsigned r = c - iz * cx * cy;
+    const unsigned iy = r / cx;
+    const int b = (int)(iz * (unsigned)sz + iy * (unsigned)sy + (r - iy * cx));
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      float a[2][8];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float *__restrict__ f = src.f[2 * p + h] + b;
+        const float v[8] = {__ldg(f),      __ldg(f + 1),      __ldg(f + sy),      __ldg(f + sy + 1),
+                            __ldg(f + sz), __ldg(f + sz + 1), __ldg(f + sz + sy), __ldg(f + sz + sy + 1)};
+        cell_coeffs(v, a[h]);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        rec[(4 * p + j) * kPackRow + lane] = make_float4(a[0][2 * j], a[1][2 * j], a[0][2 * j + 1], a[1][2 * j + 1]);
     }
+    __syncwarp();
+    float4 *dst = out + 12ull * first;
+#pragma unroll
+    for (int m = 0; m < 12; ++m) {
+      const unsigned o = lane + 32 * m;
+      if (o < 12u * n) dst[o] = rec[(o % 12u) * kPackRow + o / 12u];
+    }
+    __syncwarp();
   }
 }
 
@@ -103,8 +181,14 @@ int ap_grid_pack(const ap_grid *g, float *packed, void *stream) {
     const long long want = (cells + block - 1) / block;
     CompPtrs src;
     for (int c = 0; c < 6; ++c) src.f[c] = g->f[c];
-    pack_cells_kernel<<<(int)(want < cap ? want : cap), block, 0, s>>>(src, g->nx, g->ny, g->nz,
-                                                                      reinterpret_cast<float4 *>(packed));
+    // shared memory lets four blocks of eight warps stay resident
+    const size_t smem = sizeof(float4) * 12 * kPackRow * kPackWarps;
+    if (cudaFuncSetAttribute(pack_cells_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+        cudaSuccess)
+      return AP_ERR_CUDA;
+    const long long resident = (long long)sms * 4;
+    pack_cells_kernel<<<(int)(want < resident ? want : resident), 32 * kPackWarps, smem, s>>>(
+        src, g->nx, g->ny, g->nz, reinterpret_cast<float4 *>(packed));
   } else {
     const long long nodes = (long long)g->nx * g->ny * g->nz;
     const long long want = (nodes + block - 1) / block;
