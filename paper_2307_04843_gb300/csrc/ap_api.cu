@@ -358,6 +358,61 @@ void derive(const ap_pulse_desc &d, Pulse<double> &P, Pulse<float> &F) {
   split(P.z_f, F.zf_hi, F.zf_lo);
   split(P.ff_w, F.ffw_hi, F.ffw_lo);
   split(P.ff_dw, F.ffd_hi, F.ffd_lo);
+  // the float-float step's constants
+  apt::FastPulse &S = F.fast;
+  const double log2e = 1.4426950408889634;
+  S.z_scale = k / (2.0 * kPi);
+  S.z_len = (2.0 * kPi) / k;
+  S.frame = d.pol == AP_LIN_Y ? 1 : d.pol == AP_CIRC_M ? 2 : 0;
+  S.circ = d.pol == AP_CIRC_P || d.pol == AP_CIRC_M ? 1 : 0;
+  const double senv = P.env == AP_ENV_GAUSS ? std::sqrt(P.env_a)
+                      : P.env == AP_ENV_SIN2 || P.env == AP_ENV_SGAUSS ? P.env_a : 1.0;
+  S.s_env = (float)senv;
+  S.env_len = (float)(1.0 / senv);
+  S.env_w = (float)(P.env_a * P.env_b);
+  S.c_eta = (float)(-senv * P.inv_vg * S.z_len);
+  S.c_zn = (float)(-P.inv_zR * S.z_len);
+  S.c_tz = (float)(P.beta_f * P.inv_zR);
+  S.c_a = (float)(P.inv_w0sq * log2e);
+  double A = P.amp, ce = P.lonE * -2.0 * P.inv_w0sq, cb = P.lonB * -2.0 * P.inv_w0sq;
+  if (d.kind == AP_LG) {
+    // in the turned frame x + i sgn y = i sgn (x' + i sgn y'): |l| quarter turns
+    const double sg = (S.frame == 2 ? -1.0 : 1.0) * P.lg_sgn;
+    if (S.frame == 1) S.turn0 = 0.25 * P.lg_sgn * P.lg_al;
+    A = P.amp * P.lg_pref;
+    ce = P.lonE;
+    cb = P.lonB;
+    S.lg_sg = (float)sg;
+    S.lg_sp = (float)(1.0 + sg);
+    S.lg_m2w = (float)(-2.0 * P.inv_w0sq);
+    S.lg_m4w = (float)(-4.0 * P.inv_w0sq);
+    for (int r = 0; r < 6; ++r)
+      for (int i = 0; i < apt::kLgMaxP; ++i) S.lg_n[r][i] = (float)(r % 3 == 0 ? P.lg_r[r][i] : -P.lg_r[r][i]);
+  }
+  S.A = (float)A;
+  S.Abr = (float)(A * P.bratio);
+  S.Ace = P.lon ? (float)(A * ce) : 0.0f;
+  S.Acb = P.lon ? (float)(A * P.bratio * cb) : 0.0f;
+  if (d.kind == AP_FLYING_SUM) {
+    split(P.ff_w / P.omega, S.r0_hi, S.r0_lo);
+    split(P.ff_dw / P.omega, S.rd_hi, S.rd_lo);
+    double cmax = 0.0;
+    for (int j = 0; j < P.n_comp; ++j) {
+      const double cz = -P.comp[j].inv_zR * S.z_len;
+      double th = std::atan2(P.comp[j].c_im, P.comp[j].c_re) / (2.0 * kPi);
+      if (P.amp < 0.0) th += 0.5;  // c_j = A e^{i theta_j}
+      // a 32-bit fraction of a turn, half a turn added (the step takes the
+      // fraction less one half) and half the last of the 23 bits it keeps
+      th -= std::floor(th);
+      const uint32_t bits = (uint32_t)(uint64_t)std::llround(th * 4294967296.0) + 0x80000000u + 0x100u;
+      float4 c = make_float4((float)cz, (float)P.comp[j].zoff, 0.0f, (float)P.comp[j].inv_k);
+      std::memcpy(&c.z, &bits, sizeof(bits));
+      F.fcomp[j] = c;
+      cmax = std::max(cmax, std::fabs(cz));
+    }
+    S.z_max = (float)(1e9 / cmax);
+  }
+  P.fast = S;
   P.k_hi = F.k_hi; P.k_lo = F.k_lo; P.zf_hi = F.zf_hi; P.zf_lo = F.zf_lo;
   P.ffw_hi = F.ffw_hi; P.ffw_lo = F.ffw_lo; P.ffd_hi = F.ffd_hi; P.ffd_lo = F.ffd_lo;
 }

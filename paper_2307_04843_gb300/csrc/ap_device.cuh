@@ -892,11 +892,8 @@ __device__ __forceinline__ void grid_slots_init(GridSlots &gc, void *slots_base)
 }
 
 // Every lane of the warp calls this together (warp-uniform refetch branch).
-__device__ __forceinline__ void grid_fetch(const GridView &g, GridSlots &gc, float x, float y,
-                                           float z) {
-  const float fx = grid_unit<float>(x, g.inv_d[0], g.off[0], g.top[0]);
-  const float fy = grid_unit<float>(y, g.inv_d[1], g.off[1], g.top[1]);
-  const float fz = grid_unit<float>(z, g.inv_d[2], g.off[2], g.top[2]);
+__device__ __forceinline__ void grid_fetch_units(const GridView &g, GridSlots &gc, float fx, float fy,
+                                                 float fz) {
   float wx = fx - gc.ox, wy = fy - gc.oy, wz = fz - gc.oz;
   // inside the cached cell (faces included) iff max |w - 1/2| <= 1/2
   const float dev = fmaxf(fabsf(wx - 0.5f), fmaxf(fabsf(wy - 0.5f), fabsf(wz - 0.5f)));
@@ -939,13 +936,15 @@ __device__ __forceinline__ void grid_fetch(const GridView &g, GridSlots &gc, flo
   gc.wz = wz;
 }
 
-__device__ __forceinline__ void grid_eval(const GridSlots &gc, float E[3], float B[3]) {
-  cp_async_wait_all();  // this thread's copies (if any) have landed
+// the six interpolated components from the cached corners (the caller has
+// waited for the copies)
+__device__ __forceinline__ void grid_values(const GridSlots &gc, float o[6]) {
   const float ux = 1.0f - gc.wx, uy = 1.0f - gc.wy, uz = 1.0f - gc.wz;
   const float a00 = ux * uy, a10 = gc.wx * uy, a01 = ux * gc.wy, a11 = gc.wx * gc.wy;
   const float w[8] = {a00 * uz, a10 * uz, a01 * uz, a11 * uz, a00 * gc.wz, a10 * gc.wz,
                       a01 * gc.wz, a11 * gc.wz};
-  float o[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+  for (int c = 0; c < 6; ++c) o[c] = 0.0f;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const float4 lo = lds128(gc.s0 + (2 * k) * gc.step);
@@ -957,6 +956,12 @@ __device__ __forceinline__ void grid_eval(const GridSlots &gc, float E[3], float
     o[4] = fmaf(w[k], hi.x, o[4]);
     o[5] = fmaf(w[k], hi.y, o[5]);
   }
+}
+
+__device__ __forceinline__ void grid_eval(const GridSlots &gc, float E[3], float B[3]) {
+  cp_async_wait_all();  // this thread's copies (if any) have landed
+  float o[6];
+  grid_values(gc, o);
   E[0] += o[0]; E[1] += o[1]; E[2] += o[2];
   B[0] += o[3]; B[1] += o[4]; B[2] += o[5];
 }
@@ -1047,11 +1052,8 @@ __device__ __forceinline__ void cell_refetch(const GridView &g, CellSlots &gc, f
 }
 
 // Every lane of the warp calls this together (warp-uniform refetch branch).
-__device__ __forceinline__ void grid_fetch(const GridView &g, CellSlots &gc, float x, float y,
-                                           float z) {
-  const float fx = grid_unit<float>(x, g.inv_d[0], g.off[0], g.top[0]);
-  const float fy = grid_unit<float>(y, g.inv_d[1], g.off[1], g.top[1]);
-  const float fz = grid_unit<float>(z, g.inv_d[2], g.off[2], g.top[2]);
+__device__ __forceinline__ void grid_fetch_units(const GridView &g, CellSlots &gc, float fx, float fy,
+                                                 float fz) {
   float wx = fx - gc.ox, wy = fy - gc.oy, wz = fz - gc.oz;
   // inside the cached cell (faces included) iff max |w - 1/2| <= 1/2
   const float dev = fmaxf(fabsf(wx - 0.5f), fmaxf(fabsf(wy - 0.5f), fabsf(wz - 0.5f)));
@@ -1103,11 +1105,8 @@ __device__ __forceinline__ void cell_refetch(const GridView &g, CellRegs &gc, fl
   for (int k = 0; k < 12; ++k) gc.c[k] = __ldg(src + k);
 }
 
-__device__ __forceinline__ void grid_fetch(const GridView &g, CellRegs &gc, float x, float y,
-                                           float z) {
-  const float fx = grid_unit<float>(x, g.inv_d[0], g.off[0], g.top[0]);
-  const float fy = grid_unit<float>(y, g.inv_d[1], g.off[1], g.top[1]);
-  const float fz = grid_unit<float>(z, g.inv_d[2], g.off[2], g.top[2]);
+__device__ __forceinline__ void grid_fetch_units(const GridView &g, CellRegs &gc, float fx, float fy,
+                                                 float fz) {
   float wx = fx - gc.ox, wy = fy - gc.oy, wz = fz - gc.oz;
   // inside the cached cell (faces included) iff max |w - 1/2| <= 1/2
   const float dev = fmaxf(fabsf(wx - 0.5f), fmaxf(fabsf(wy - 0.5f), fabsf(wz - 0.5f)));
@@ -1116,6 +1115,14 @@ __device__ __forceinline__ void grid_fetch(const GridView &g, CellRegs &gc, floa
   gc.wx = wx;
   gc.wy = wy;
   gc.wz = wz;
+}
+
+// from a position: its grid units, then the fetch
+template <class GC>
+__device__ __forceinline__ void grid_fetch_at(const GridView &g, GC &gc, float x, float y, float z) {
+  grid_fetch_units(g, gc, grid_unit<float>(x, g.inv_d[0], g.off[0], g.top[0]),
+                   grid_unit<float>(y, g.inv_d[1], g.off[1], g.top[1]),
+                   grid_unit<float>(z, g.inv_d[2], g.off[2], g.top[2]));
 }
 
 __device__ __forceinline__ void grid_values(const CellRegs &gc, float o[6]) {

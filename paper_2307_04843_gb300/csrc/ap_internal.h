@@ -27,10 +27,29 @@ struct Comp {
   R c_re, c_im;
 };
 
+// Constants of the float-float step (ap_step.cuh), which carries the
+// longitudinal position in turns of the carrier, Z = k (z - z_f) / 2 pi, and
+// runs y-polarised and left-handed pulses in a turned or mirrored frame.
+struct FastPulse {
+  double z_scale, z_len;  // k / 2 pi and 2 pi / k
+  double turn0;           // carrier phase that the frame adds (turns)
+  float s_env, env_len;   // scale of the envelope argument, and its inverse
+  float env_w;            // half-width of the sin^2 window, scaled
+  float c_eta, c_zn, c_tz;  // eta s_env = s_env T + c_eta Z, -zeta = c_zn Z + c_tz T
+  float c_a;              // log2(e) / w0^2
+  float A, Abr, Ace, Acb;  // E_perp, B_perp, E_z, B_z per unit field
+  float lg_n[6][kLgMaxP];  // the Laguerre recurrences with the subtracted terms' signs in
+  float lg_sg, lg_sp, lg_m2w, lg_m4w;  // sgn l, 1 + sgn l (in the frame), -2/w0^2, -4/w0^2
+  float r0_hi, r0_lo, rd_hi, rd_lo;    // flying focus: w_first / omega, dw / omega
+  float z_max;            // |Z| beyond which every |zeta_j| > 1e9
+  int32_t frame;          // 0: none, 1: x' = y, y' = -x, 2: y' = -y
+  int32_t circ;           // circular polarisation
+};
+
 // Device-side description of one pulse, derived on the host in FP64 (row a1)
 // and rounded once to the arithmetic type R of the push.
 template <typename R>
-struct Pulse {
+struct PulseHead {
   static constexpr bool kHasPlasma = true;  // carries the Sec. 4 plasma constants
   int32_t kind, pol, env, lon;
   int32_t lg_p, lg_al, lg_sgn, n_comp;
@@ -66,7 +85,16 @@ struct Pulse {
   // float-float copies for AP_FP32_PHASEFF
   double ff_w, ff_dw;
   float ffw_hi, ffw_lo, ffd_hi, ffd_lo;
+  FastPulse fast;
+};
+
+// The component tables only the flying-focus sum needs: comp for the generic
+// field code; fcomp for the float-float step, {-2 pi / (k z_R,j), zoff_j, phase
+// as the bits of a 32-bit fraction of a turn, 1/k_j}.
+template <typename R>
+struct Pulse : PulseHead<R> {
   Comp<R> comp[kMaxComp];
+  float4 fcomp[kMaxComp];
 };
 
 // Grid view passed to kernels (device pointers, caller-owned).

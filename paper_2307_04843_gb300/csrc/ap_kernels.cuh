@@ -5,7 +5,7 @@
 
 #include <type_traits>
 
-#include "ap_pair.cuh"
+#include "ap_step.cuh"
 
 namespace apt {
 
@@ -68,19 +68,17 @@ __host__ __device__ constexpr size_t grid_cache_bytes(int threads) {
                                                                       : grid_slot_bytes(threads);
 }
 
-// One particle through n_steps fused steps: load (a2), per step the local
-// coordinates and phase (a3), envelope and profile (a4-a7), grid gather
-// (a8), Boris and position (a9), light-front diagnostic (a10); then store
-// (a11).  Every lane of a warp calls this together: the float-float variant
-// tabulates the per-step phase base C_n and time T_n for its warp in shared
-// memory, 32 steps at a time (one entry per lane, __syncwarp only, so warps
-// never wait for each other).  `valid` is false for padding threads, which
-// run the loop on a dummy particle so that warp operations see every lane.
-// Returns the final gamma (double) of a valid particle, 0 otherwise.
+// One particle through n_steps fused steps in double or with native double
+// phase and position: load (a2), per step the local coordinates and phase
+// (a3), envelope and profile (a4-a7), grid gather (a8), Boris and position
+// (a9), light-front diagnostic (a10); then store (a11).  Every lane of a warp
+// calls this together; `valid` is false for padding threads, which run the
+// loop on a dummy particle so that warp operations see every lane.  Returns
+// the final gamma (double) of a valid particle, 0 otherwise.
 template <int KIND, int PREC, int GRID>
-__device__ __forceinline__ double push_one(const Pulse<Real<PREC>> &P, const PushArgs &a,
-                                           long long i, bool valid, StepFF *s_steps,
+__device__ __forceinline__ double push_one(const Pulse<Real<PREC>> &P, const PushArgs &a, long long i, bool valid,
                                            void *slots) {
+  static_assert(PREC != AP_FP32_PHASEFF, "push_ff");
   using R = Real<PREC>;
   double X = 0.0, Y = 0.0, Z = 0.0;
   R u[3] = {R(0), R(0), R(0)};
@@ -106,34 +104,23 @@ __device__ __forceinline__ double push_one(const Pulse<Real<PREC>> &P, const Pus
   if constexpr (GRID && !std::is_same<R, double>::value) grid_slots_init(gc, slots);
   else grid_cache_reset(gc);
   double *lf = a.diag.lf;
-  StepFF *wsteps = s_steps + (threadIdx.x >> 5) * kStepChunk;
-  const int lane = threadIdx.x & 31;
   // the step loop, compiled twice: with the per-step light-front diagnostic
   // and without it (its test would otherwise cost every step an issue slot)
   auto steps = [&](auto with_lf) {
     constexpr bool LF = decltype(with_lf)::value;
-    for (long long s0 = 0; s0 < a.n_steps; s0 += kStepChunk) {
-      const int cnt = (int)(a.n_steps - s0 < kStepChunk ? a.n_steps - s0 : kStepChunk);
-      if constexpr (PREC == AP_FP32_PHASEFF) {
-        __syncwarp();  // no lane still reads the previous chunk
-        if (lane < cnt) wsteps[lane] = tb.at(s0 + lane);
-        __syncwarp();
-      }
-      for (int k = 0; k < cnt; ++k) {
-        typename TimeBase<PREC>::Step st;
-        if constexpr (PREC == AP_FP32_PHASEFF) st = wsteps[k];
-        else st = tb.at(s0 + k);
-        Local<R> L = local_coords<PREC>(P, st, pos);
-        if constexpr (GRID) grid_fetch(a.grid, gc, L.x, L.y, pos.zr());
-        R E[3], B[3];
-        analytic_fields<KIND, PREC>(P, L, E, B);
-        if constexpr (GRID) grid_eval(gc, E, B);
-        R ig = boris(u, E, B, dtR);
-        pos.advance(u[0] * ig, u[1] * ig, u[2] * ig, dtxy, dtR);
-        if constexpr (LF) {
-          R dev = valid ? fabs((R(1) / ig - u[2]) - h0) : R(0);
-          warp_max_to(lf + s0 + k, dev, 0xffffffffu);
-        }
+    for (long long n = 0; n < a.n_steps; ++n) {
+      const typename TimeBase<PREC>::Step st = tb.at(n);
+      Local<R> L = local_coords<PREC>(P, st, pos);
+      if constexpr (GRID && std::is_same<R, double>::value) grid_fetch(a.grid, gc, L.x, L.y, pos.zr());
+      else if constexpr (GRID) grid_fetch_at(a.grid, gc, L.x, L.y, pos.zr());
+      R E[3], B[3];
+      analytic_fields<KIND, PREC>(P, L, E, B);
+      if constexpr (GRID) grid_eval(gc, E, B);
+      R ig = boris(u, E, B, dtR);
+      pos.advance(u[0] * ig, u[1] * ig, u[2] * ig, dtxy, dtR);
+      if constexpr (LF) {
+        R dev = valid ? fabs((R(1) / ig - u[2]) - h0) : R(0);
+        warp_max_to(lf + n, dev, 0xffffffffu);
       }
     }
   };
@@ -155,134 +142,259 @@ __device__ __forceinline__ double push_one(const Pulse<Real<PREC>> &P, const Pus
                               1.0));
 }
 
-// Two particles per thread (float-float variant, grid none or per-cell
-// coefficients in registers): particle i0 rides in the low half and i1 in the
-// high half of every packed value (ap_pair.cuh), so each FP32 instruction of
-// the local coordinates, the field, the Boris step and the position update
-// serves both.  The steps and their order are those of push_one; each
-// particle keeps its own grid cell (its refetch is its own warp-uniform
-// branch) and the cell is evaluated with packed FMA over component pairs.
-// `v0`, `v1` are false for padding particles.  g receives the final gammas.
-// The block's pre-broadcast grid constants for grid_fetch2 (written by the
-// first four threads; the caller synchronises the block before use).
-__device__ __forceinline__ void grid_pair_consts(const GridView &g, float4 *gk) {
+// One or two particles of a thread (R = float or F2) through n_steps fused
+// float-float steps (ap_step.cuh): load (a2), per step the phase and unit
+// fields (a3-a7), grid gather (a8), Boris and position (a9), light-front
+// diagnostic (a10); then store (a11).  With two, particle i0 rides in the low
+// half and i1 in the high half of every packed value, so each FP32
+// instruction serves both; each keeps its own grid cell (its refetch is its
+// own warp-uniform branch).  Every lane of a warp calls this together: the
+// step table (phase C_n and time T_n) is made for the warp in shared memory
+// 32 steps at a time, one entry per lane, __syncwarp only, so warps never
+// wait for each other.  `v0`, `v1` are false for padding particles, which run
+// the loop on a dummy state.  g receives the final gammas.
+//
+// Without a grid the pulse's frame is applied on load and store (y-polarised:
+// x' = y, y' = -x; left-handed: y' = -y), so the loop knows two polarisations.
+// With a grid the particles stay in the grid's frame and the analytic field
+// is turned into it.  The loop is compiled for the common combinations (linear
+// with a Gaussian envelope; linear; circular) and with and without the
+// light-front test, which would otherwise cost every step its branches.
+
+// grid units of the coordinates, and the thread's constants of grid_fetch2:
+// written by the first four threads; the caller synchronises the block before
+// use
+__device__ __forceinline__ void grid_pair_consts(const GridView &g, const StepBase &s, float4 *gk) {
   if (threadIdx.x < 3) {
     const int ax = threadIdx.x;
-    gk[ax] = make_float4(g.inv_d[ax], g.inv_d[ax], g.off[ax], g.off[ax]);
+    const float f = ax == 2 ? s.gz_s : g.inv_d[ax], o = ax == 2 ? s.gz_o : g.off[ax];
+    gk[ax] = make_float4(f, f, o, o);
   } else if (threadIdx.x == 3) {
     gk[3] = make_float4(0.5f, 0.5f, 0.0f, 0.0f);
   }
 }
 
-template <int KIND, int GRID>
-__device__ __forceinline__ void push_two(const Pulse<float> &P, const PushArgs &a, long long i0,
-                                         long long i1, bool v0, bool v1, StepFF *s_steps,
-                                         void *slots, const float4 *gk, double g[2]) {
-  static_assert(GRID == kGridNone || GRID == kGridCells || GRID == kGridCellsReg ||
-                    GRID == kGridCellsMix,
-                "two-particle grid modes");
-  double X[2] = {0.0, 0.0}, Y[2] = {0.0, 0.0}, Z[2] = {0.0, 0.0};
-  float ua[3] = {0.0f, 0.0f, 0.0f}, ub[3] = {0.0f, 0.0f, 0.0f};
-  {
-    const float *ux = static_cast<const float *>(a.ux);
-    const float *uy = static_cast<const float *>(a.uy);
-    const float *uz = static_cast<const float *>(a.uz);
-    if (v0) {
-      X[0] = a.x[i0]; Y[0] = a.y[i0]; Z[0] = a.z[i0];
-      ua[0] = ux[i0]; ua[1] = uy[i0]; ua[2] = uz[i0];
-    }
-    if (v1) {
-      X[1] = a.x[i1]; Y[1] = a.y[i1]; Z[1] = a.z[i1];
-      ub[0] = ux[i1]; ub[1] = uy[i1]; ub[2] = uz[i1];
+// the cell caches of a thread's one or two particles
+template <int GRID, typename R>
+struct Caches {
+  using A = typename CacheOf<AP_FP32_PHASEFF, GRID>::type;
+  A a;
+  __device__ __forceinline__ void init(void *slots) {
+    if constexpr (GRID != kGridNone) grid_slots_init(a, slots);
+  }
+  __device__ __forceinline__ void fetch(const GridView &g, const StepBase &s, const float4 *, R x, R y, R zhi) {
+    grid_fetch_units(g, a, grid_unit<float>(x, g.inv_d[0], g.off[0], g.top[0]),
+                     grid_unit<float>(y, g.inv_d[1], g.off[1], g.top[1]),
+                     grid_unit<float>(zhi, s.gz_s, s.gz_o, g.top[2]));
+  }
+  __device__ __forceinline__ void values(R G[6]) {
+    if constexpr (GRID != kGridCellsReg) cp_async_wait_all();  // this thread's copies landed
+    grid_values(a, G);
+  }
+};
+template <int GRID>
+struct Caches<GRID, F2> {
+  using A = typename std::conditional<GRID == kGridCells, CellSlots, CellRegs>::type;
+  using B = typename std::conditional<GRID == kGridCellsReg, CellRegs, CellSlots>::type;
+  A a;
+  B b;
+  __device__ __forceinline__ void init(void *slots) {
+    if constexpr (GRID == kGridCellsMix) {
+      grid_slots_init(a, nullptr);
+      grid_slots_init(b, slots);
+    } else if constexpr (GRID != kGridNone) {
+      grid_slots_init(a, slots);
+      grid_slots_init(b, static_cast<unsigned char *>(slots) + 12u * kCellSlotStride);
     }
   }
-  F2 u[3] = {F2(ua[0], ub[0]), F2(ua[1], ub[1]), F2(ua[2], ub[2])};
-  Pos2 pos;
-  pos.load(X, Y, Z, P.z_f);
-  TimeBase<AP_FP32_PHASEFF> tb;
-  tb.init(P, a.t0, a.dt);
-  const float dts = (float)a.dt;
-  const F2 dtR = dts, dtxy = dts * P.adv_xy;
-  // light-front reference h0 = gamma - u_z on entry, per particle as in push_one
-  const float h0a = 1.0f / rsqrt_r(fmaf(ua[0], ua[0], fmaf(ua[1], ua[1], fmaf(ua[2], ua[2], 1.0f)))) - ua[2];
-  const float h0b = 1.0f / rsqrt_r(fmaf(ub[0], ub[0], fmaf(ub[1], ub[1], fmaf(ub[2], ub[2], 1.0f)))) - ub[2];
-  // cell caches: registers, or two regions of the block's shared slots (the
-  // second particle's 12 slots per thread after the first's)
-  using CacheA = typename std::conditional<GRID == kGridCells, CellSlots, CellRegs>::type;
-  using CacheB = typename std::conditional<GRID == kGridCellsReg, CellRegs, CellSlots>::type;
-  CacheA gca;
-  CacheB gcb;
-  if constexpr (GRID == kGridCellsMix) {
-    grid_slots_init(gca, nullptr);
-    grid_slots_init(gcb, slots);
-  } else if constexpr (GRID != kGridNone) {
-    grid_slots_init(gca, slots);
-    grid_slots_init(gcb, static_cast<unsigned char *>(slots) + 12u * kCellSlotStride);
+  __device__ __forceinline__ void fetch(const GridView &g, const StepBase &, const float4 *gk, F2 x, F2 y, F2 zhi) {
+    grid_fetch2(g, a, b, x, y, zhi, gk);
   }
+  __device__ __forceinline__ void values(F2 G[6]) {
+    if constexpr (GRID != kGridCellsReg) cp_async_wait_all();
+    float oa[6], ob[6];
+    grid_values(a, oa);
+    grid_values(b, ob);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) G[c] = F2(oa[c], ob[c]);
+  }
+};
+
+// grid value plus factor times unit field, by scalar operations (the two
+// particles' grid values come from different register pairs)
+__device__ __forceinline__ float grid_plus(float f, float u, float g) { return rfma(f, u, g); }
+__device__ __forceinline__ F2 grid_plus(float f, F2 u, F2 g) { return F2(rfma(f, u.x, g.x), rfma(f, u.y, g.y)); }
+
+template <typename R>
+__device__ __forceinline__ R pack_lanes(float a, float b) {
+  if constexpr (IsPair<R>::value) return R(a, b);
+  else return a;
+}
+__device__ __forceinline__ float lane_of(float v, int) { return v; }
+__device__ __forceinline__ float lane_of(F2 v, int h) { return h ? v.y : v.x; }
+
+template <int KIND, int GRID, typename R, class PT>
+__device__ __forceinline__ void push_ff(const PT &P, const StepBase &sb, const PushArgs &a, long long i0, long long i1,
+                                        bool v0, bool v1, float4 *s_steps, const float4 *comps, void *slots,
+                                        const float4 *gk, double g[2]) {
+  using FFR = typename FFOf<R>::type;
+  constexpr int NP = IsPair<R>::value ? 2 : 1;
+  const FastPulse &F = P.fast;
+  const long long idx[2] = {i0, i1};
+  const bool val[2] = {v0, v1};
+  const int frame = GRID == kGridNone ? F.frame : 0;
+  FF px[2], py[2], pz[2];
+  float uu[2][3], h0[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    px[h] = py[h] = pz[h] = FF{0.0f, 0.0f};
+    uu[h][0] = uu[h][1] = uu[h][2] = 0.0f;
+    if (h < NP && val[h]) {
+      const long long i = idx[h];
+      px[h] = split_double(a.x[i]);
+      py[h] = split_double(a.y[i]);
+      pz[h] = split_double(__dmul_rn(__dsub_rn(a.z[i], P.z_f), F.z_scale));
+      uu[h][0] = static_cast<const float *>(a.ux)[i];
+      uu[h][1] = static_cast<const float *>(a.uy)[i];
+      uu[h][2] = static_cast<const float *>(a.uz)[i];
+      if (frame == 1) {
+        const FF t = px[h];
+        px[h] = py[h];
+        py[h] = FF{-t.hi, -t.lo};
+        const float tu = uu[h][0];
+        uu[h][0] = uu[h][1];
+        uu[h][1] = -tu;
+      } else if (frame == 2) {
+        py[h] = FF{-py[h].hi, -py[h].lo};
+        uu[h][1] = -uu[h][1];
+      }
+    }
+    // light-front reference h0 = gamma - u_z on entry
+    h0[h] = 1.0f / rsqrt_r(fmaf(uu[h][0], uu[h][0], fmaf(uu[h][1], uu[h][1], fmaf(uu[h][2], uu[h][2], 1.0f)))) -
+            uu[h][2];
+  }
+  FFR x{pack_lanes<R>(px[0].hi, px[1].hi), pack_lanes<R>(px[0].lo, px[1].lo)};
+  FFR y{pack_lanes<R>(py[0].hi, py[1].hi), pack_lanes<R>(py[0].lo, py[1].lo)};
+  FFR z{pack_lanes<R>(pz[0].hi, pz[1].hi), pack_lanes<R>(pz[0].lo, pz[1].lo)};
+  R u[3] = {pack_lanes<R>(uu[0][0], uu[1][0]), pack_lanes<R>(uu[0][1], uu[1][1]), pack_lanes<R>(uu[0][2], uu[1][2])};
+  Caches<GRID, R> gc;
+  gc.init(slots);
   double *lf = a.diag.lf;
-  StepFF *wsteps = s_steps + (threadIdx.x >> 5) * kStepChunk;
+  float4 *wsteps = s_steps + (threadIdx.x >> 5) * kStepChunk;
   const int lane = threadIdx.x & 31;
-  auto steps = [&](auto with_lf) {
-    constexpr bool LF = decltype(with_lf)::value;
+
+  auto steps = [&](auto pol_c, auto env_c, auto lf_c) {
+    constexpr int POL = decltype(pol_c)::value, ENV = decltype(env_c)::value;
+    constexpr bool LF = decltype(lf_c)::value;
     for (long long s0 = 0; s0 < a.n_steps; s0 += kStepChunk) {
       const int cnt = (int)(a.n_steps - s0 < kStepChunk ? a.n_steps - s0 : kStepChunk);
       __syncwarp();  // no lane still reads the previous chunk
-      if (lane < cnt) wsteps[lane] = tb.at(s0 + lane);
+      if (lane < cnt) wsteps[lane] = step_entry<KIND>(F, sb, (float)(int)(s0 + lane));
       __syncwarp();
 #pragma unroll 2
       for (int k = 0; k < cnt; ++k) {
-        const StepFF st = wsteps[k];
-        const Local<F2> L = local_coords2(P, st, pos);
-        if constexpr (GRID != kGridNone)
-          grid_fetch2(a.grid, gca, gcb, L.x, L.y, pos.zr(P.zf_hi, P.zf_lo), gk);
-        F2 E[3], B[3];
-        analytic_fields<KIND, AP_FP32_PHASEFF, F2>(P, L, E, B);
-        if constexpr (GRID != kGridNone) {
-          if constexpr (GRID == kGridCells || GRID == kGridCellsMix)
-            cp_async_wait_all();  // this thread's copies landed
-          float oa[6], ob[6];
-          grid_values(gca, oa);
-          grid_values(gcb, ob);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            E[c].x += oa[c]; E[c].y += ob[c];
-            B[c].x += oa[c + 3]; B[c].y += ob[c + 3];
+        const float4 st = wsteps[k];
+        R ig;
+        if constexpr (GRID == kGridNone) {
+          const UnitFields<R> f = unit_fields<KIND, POL, ENV>(P, comps, st, x.hi, y.hi, z.hi, z.lo);
+          ig = boris_unit<POL, KIND != AP_PLANE>(u, f, sb);
+        } else {
+          gc.fetch(a.grid, sb, gk, x.hi, y.hi, z.hi);
+          R xe = x.hi, ye = y.hi;
+          if constexpr (ENV == kEnvAny) {  // the common case has no frame
+            if (F.frame == 1) {
+              xe = y.hi;
+              ye = rneg(x.hi);
+            } else if (F.frame == 2) {
+              ye = rneg(y.hi);
+            }
           }
+          const UnitFields<R> f = unit_fields<KIND, POL, ENV>(P, comps, st, xe, ye, z.hi, z.lo);
+          R G[6];
+          gc.values(G);
+          if (POL == kLin) {
+            if (ENV == kEnvGauss || F.frame == 0) {
+              G[0] = grid_plus(F.A, f.Ur, G[0]);
+              G[4] = grid_plus(F.Abr, f.Vr, G[4]);
+            } else {
+              G[1] = grid_plus(F.A, f.Ur, G[1]);
+              G[3] = grid_plus(-F.Abr, f.Vr, G[3]);
+            }
+            G[2] = grid_plus(F.Ace, f.ez, G[2]);
+            G[5] = grid_plus(F.Acb, f.bz, G[5]);
+          } else {
+            const float sg = F.frame == 2 ? -1.0f : 1.0f;  // exact signs
+            G[0] = grid_plus(F.A, f.Ur, G[0]);
+            G[1] = grid_plus(sg * F.A, f.Ui, G[1]);
+            G[2] = grid_plus(F.Ace, f.ez, G[2]);
+            G[3] = grid_plus(-sg * F.Abr, f.Vi, G[3]);
+            G[4] = grid_plus(F.Abr, f.Vr, G[4]);
+            G[5] = grid_plus(sg * F.Acb, f.bz, G[5]);
+          }
+          ig = boris_full(u, G, G + 3, sb.h, sb.k);
         }
-        const F2 ig = boris(u, E, B, dtR);
-        pos.advance(u[0] * ig, u[1] * ig, u[2] * ig, dtxy, dtR);
+        const R kxy = rmul(R(sb.cxy), ig);
+        advance(x, u[0], kxy);
+        advance(y, u[1], kxy);
+        advance(z, u[2], rmul(R(sb.cz), ig));
         if constexpr (LF) {
-          const float da = v0 ? fabsf((1.0f / ig.x - u[2].x) - h0a) : 0.0f;
-          const float db = v1 ? fabsf((1.0f / ig.y - u[2].y) - h0b) : 0.0f;
-          warp_max_to(lf + s0 + k, fmaxf(da, db), 0xffffffffu);
+          float dev = 0.0f;
+#pragma unroll
+          for (int h = 0; h < NP; ++h)
+            if (val[h]) dev = fmaxf(dev, fabsf((1.0f / lane_of(ig, h) - lane_of(u[2], h)) - h0[h]));
+          warp_max_to(lf + s0 + k, dev, 0xffffffffu);
         }
       }
     }
   };
-  if (lf) steps(std::true_type{});
-  else steps(std::false_type{});
-  const long long idx[2] = {i0, i1};
-  const bool val[2] = {v0, v1};
+  using Lin = std::integral_constant<int, kLin>;
+  using Circ = std::integral_constant<int, kCirc>;
+  using EnvG = std::integral_constant<int, kEnvGauss>;
+  using EnvA = std::integral_constant<int, kEnvAny>;
+  // kinds without an envelope switch or with no Gaussian default take the
+  // general loop
+  constexpr bool kGaussLoop = KIND == AP_GAUSS || KIND == AP_FLYING_CF;
+  if (lf) {
+    if (F.circ) steps(Circ{}, EnvA{}, std::true_type{});
+    else steps(Lin{}, EnvA{}, std::true_type{});
+  } else if (F.circ) {
+    steps(Circ{}, EnvA{}, std::false_type{});
+  } else if (kGaussLoop && P.env == AP_ENV_GAUSS && (GRID == kGridNone || F.frame == 0)) {
+    if constexpr (kGaussLoop) steps(Lin{}, EnvG{}, std::false_type{});
+  } else {
+    steps(Lin{}, EnvA{}, std::false_type{});
+  }
+
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < NP; ++h) {
     g[h] = 0.0;
     if (!val[h]) continue;
     const long long i = idx[h];
-    const FF px{h ? pos.x.hi.y : pos.x.hi.x, h ? pos.x.lo.y : pos.x.lo.x};
-    const FF py{h ? pos.y.hi.y : pos.y.hi.x, h ? pos.y.lo.y : pos.y.lo.x};
-    const FF pz{h ? pos.dz.hi.y : pos.dz.hi.x, h ? pos.dz.lo.y : pos.dz.lo.x};
-    a.x[i] = (double)px.hi + (double)px.lo;
-    a.y[i] = (double)py.hi + (double)py.lo;
-    a.z[i] = ((double)pz.hi + (double)pz.lo) + P.z_f;
-    const float fu[3] = {h ? u[0].y : u[0].x, h ? u[1].y : u[1].x, h ? u[2].y : u[2].x};
+    double X = (double)lane_of(x.hi, h) + (double)lane_of(x.lo, h);
+    double Y = (double)lane_of(y.hi, h) + (double)lane_of(y.lo, h);
+    const double Z = __dadd_rn(__dmul_rn((double)lane_of(z.hi, h) + (double)lane_of(z.lo, h), F.z_len), P.z_f);
+    float fu[3] = {lane_of(u[0], h), lane_of(u[1], h), lane_of(u[2], h)};
+    if (frame == 1) {
+      const double t = X;
+      X = -Y;
+      Y = t;
+      const float tu = fu[0];
+      fu[0] = -fu[1];
+      fu[1] = tu;
+    } else if (frame == 2) {
+      Y = -Y;
+      fu[1] = -fu[1];
+    }
+    a.x[i] = X;
+    a.y[i] = Y;
+    a.z[i] = Z;
     static_cast<float *>(a.ux)[i] = fu[0];
     static_cast<float *>(a.uy)[i] = fu[1];
     static_cast<float *>(a.uz)[i] = fu[2];
     const double dx = (double)fu[0], dy = (double)fu[1], dz = (double)fu[2];
-    if (!all_finite(a.x[i], a.y[i], a.z[i], dx, dy, dz)) atomicOr(a.status, kStatusNonfinite);
-    g[h] = __dsqrt_rn(__dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
-                                          __dmul_rn(dz, dz)),
-                                1.0));
+    if (!all_finite(X, Y, Z, dx, dy, dz)) atomicOr(a.status, kStatusNonfinite);
+    // gamma in double from the stored momentum, fixed operation order
+    g[h] = __dsqrt_rn(__dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)), 1.0));
   }
 }
 
@@ -306,25 +418,28 @@ __device__ __forceinline__ double block_sum(double v, double *s_red) {
   return r;
 }
 
+// The pulse a float-float kernel is given: the component tables only where
+// the kind has them.
+template <int KIND>
+using FFPulse = typename std::conditional<KIND == AP_FLYING_SUM, Pulse<float>, PulseHead<float>>::type;
+
+// float4 of a block's component table (one particle per thread reads 16 bytes
+// per component, two 32)
+template <int KIND, int NP>
+__host__ __device__ constexpr int comp_slots() { return KIND == AP_FLYING_SUM ? kMaxComp * NP : 1; }
+
 // Plain launch: a grid-stride loop over block-sized chunks of particles (the
-// trip count is uniform across the block), one particle per thread, every
-// step fused.  Dynamic shared memory: step tables, grid slots (float grid
-// kernels), then the histogram (hist_off bytes in).
-template <int KIND, int PREC, int GRID, int NP = 1>
-__device__ __forceinline__ void push_body(const Pulse<Real<PREC>> &P, const PushArgs &a, unsigned hist_off) {
-  extern __shared__ __align__(16) unsigned char s_dyn[];
+// trip count is uniform across the block), every step fused.  Dynamic shared
+// memory: step tables, grid slots (float grid kernels), then the histogram
+// (hist_off bytes in).  `push` advances the particles at base + threadIdx.x
+// (and, with two per thread, one block further) and returns their gammas.
+template <int NP, class Push>
+__device__ __forceinline__ void push_chunks(const PushArgs &a, unsigned char *s_dyn, unsigned hist_off, const Push &push) {
   __shared__ double s_red[32];
-  StepFF *s_steps = reinterpret_cast<StepFF *>(s_dyn);
-  void *slots = s_dyn + step_table_bytes(blockDim.x);
   uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_dyn + hist_off);
   const bool hist = a.diag.hist != nullptr;
   if (hist) {
     for (int b = threadIdx.x; b < a.diag.bins; b += blockDim.x) s_hist[b] = 0u;
-    __syncthreads();
-  }
-  __shared__ float4 s_gridk[4];
-  if constexpr (NP == 2) {
-    grid_pair_consts(a.grid, s_gridk);
     __syncthreads();
   }
   double acc = 0.0;
@@ -333,24 +448,13 @@ __device__ __forceinline__ void push_body(const Pulse<Real<PREC>> &P, const Push
   const long long stride = (long long)NP * gridDim.x * blockDim.x;
   for (long long base = (long long)NP * blockIdx.x * blockDim.x; base < a.n; base += stride) {
     const long long i = base + threadIdx.x;
-    if constexpr (NP == 2) {
-      const long long i1 = i + blockDim.x;
-      double g[2];
-      push_two<KIND, GRID>(P, a, i, i1, i < a.n, i1 < a.n, s_steps, slots, s_gridk, g);
-      if (i < a.n) {
-        acc += g[0];
-        if (hist) hist_add(s_hist, a.diag, g[0]);
-      }
-      if (i1 < a.n) {
-        acc += g[1];
-        if (hist) hist_add(s_hist, a.diag, g[1]);
-      }
-    } else {
-      const bool valid = i < a.n;
-      double g = push_one<KIND, PREC, GRID>(P, a, i, valid, s_steps, slots);
-      if (valid) {
-        acc += g;
-        if (hist) hist_add(s_hist, a.diag, g);
+    double g[2] = {0.0, 0.0};
+    push(i, g);
+#pragma unroll
+    for (int h = 0; h < NP; ++h) {
+      if (i + h * (long long)blockDim.x < a.n) {
+        acc += g[h];
+        if (hist) hist_add(s_hist, a.diag, g[h]);
       }
     }
   }
@@ -363,6 +467,33 @@ __device__ __forceinline__ void push_body(const Pulse<Real<PREC>> &P, const Push
     for (int b = threadIdx.x; b < a.diag.bins; b += blockDim.x)
       if (s_hist[b]) atomicAdd(&a.diag.hist[b], s_hist[b]);
   }
+}
+
+// double, or native double phase: one particle per thread
+template <int KIND, int PREC, int GRID>
+__device__ __forceinline__ void push_body(const Pulse<Real<PREC>> &P, const PushArgs &a, unsigned hist_off) {
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  push_chunks<1>(a, s_dyn, hist_off, [&](long long i, double g[2]) {
+    g[0] = push_one<KIND, PREC, GRID>(P, a, i, i < a.n, s_dyn + step_table_bytes(blockDim.x));
+  });
+}
+
+// float-float: NP particles per thread
+template <int KIND, int GRID, int NP>
+__device__ __forceinline__ void push_ff_body(const FFPulse<KIND> &P, const StepBase &sb, const PushArgs &a,
+                                             unsigned hist_off) {
+  using R = typename std::conditional<NP == 2, F2, float>::type;
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  __shared__ float4 s_gridk[4];
+  __shared__ float4 s_comp[comp_slots<KIND, NP>()];
+  if constexpr (KIND == AP_FLYING_SUM) comp_table<R>(P, s_comp);
+  if constexpr (NP == 2 && GRID != kGridNone) grid_pair_consts(a.grid, sb, s_gridk);
+  if constexpr (KIND == AP_FLYING_SUM || (NP == 2 && GRID != kGridNone)) __syncthreads();
+  push_chunks<NP>(a, s_dyn, hist_off, [&](long long i, double g[2]) {
+    const long long i1 = i + blockDim.x;
+    push_ff<KIND, GRID, R>(P, sb, a, i, i1, i < a.n, NP == 2 && i1 < a.n, reinterpret_cast<float4 *>(s_dyn), s_comp,
+                           s_dyn + step_table_bytes(blockDim.x), s_gridk, g);
+  });
 }
 
 // Two entries for the same body.  The per-cell coefficient variants name a
@@ -384,35 +515,33 @@ __global__ void __launch_bounds__(256, GRID == kGridCells ? 3 : 2)
   push_body<KIND, PREC, GRID>(P, a, hist_off);
 }
 
-// Two particles per thread (AP_FP32_PHASEFF; no grid, or per-cell
-// coefficients cached in shared memory or in registers).
-template <int KIND, int GRID>
-__global__ void __launch_bounds__(256)
-    push_kernel_pair(const __grid_constant__ Pulse<float> P, const __grid_constant__ PushArgs a,
-                     unsigned hist_off) {
-  push_body<KIND, AP_FP32_PHASEFF, GRID, 2>(P, a, hist_off);
-}
-// cells in shared memory: 2 resident blocks of 256 (384 B of slots per thread)
-template <int KIND>
-__global__ void __launch_bounds__(256, 2)
-    push_kernel_pair_smem(const __grid_constant__ Pulse<float> P, const __grid_constant__ PushArgs a,
-                          unsigned hist_off) {
-  push_body<KIND, AP_FP32_PHASEFF, kGridCells, 2>(P, a, hist_off);
-}
-// first cell in registers, second in shared memory: 2 resident blocks of 256
-// (128 registers, 192 B of slots per thread)
-template <int KIND>
-__global__ void __launch_bounds__(256, 2)
-    push_kernel_pair_mix(const __grid_constant__ Pulse<float> P, const __grid_constant__ PushArgs a,
-                         unsigned hist_off) {
-  push_body<KIND, AP_FP32_PHASEFF, kGridCellsMix, 2>(P, a, hist_off);
-}
-
-
 template <int KIND, int PREC, int GRID>
 constexpr auto push_entry() {
   if constexpr (GRID == kGridCells || GRID == kGridCellsReg) return push_kernel_cells<KIND, PREC, GRID>;
   else return push_kernel<KIND, PREC, GRID>;
+}
+
+// float-float: without a residency target, and with one (blocks of 256 per
+// SM: 3 for one particle per thread with its cell in shared memory, 2 with it
+// in registers or with two particles per thread and a cell in shared memory)
+template <int KIND, int GRID, int NP>
+__global__ void __launch_bounds__(256)
+    push_ff_kernel(const __grid_constant__ FFPulse<KIND> P, const __grid_constant__ StepBase sb,
+                   const __grid_constant__ PushArgs a, unsigned hist_off) {
+  push_ff_body<KIND, GRID, NP>(P, sb, a, hist_off);
+}
+template <int KIND, int GRID, int NP>
+__global__ void __launch_bounds__(256, NP == 1 && GRID == kGridCells ? 3 : 2)
+    push_ff_kernel_cells(const __grid_constant__ FFPulse<KIND> P, const __grid_constant__ StepBase sb,
+                         const __grid_constant__ PushArgs a, unsigned hist_off) {
+  push_ff_body<KIND, GRID, NP>(P, sb, a, hist_off);
+}
+
+template <int KIND, int GRID, int NP>
+constexpr auto push_ff_entry() {
+  if constexpr (GRID == kGridCells || GRID == kGridCellsMix || (GRID == kGridCellsReg && NP == 1))
+    return push_ff_kernel_cells<KIND, GRID, NP>;
+  else return push_ff_kernel<KIND, GRID, NP>;
 }
 
 // Batched persistent launch (row a12): blocks pop fixed-size tiles of
@@ -421,38 +550,57 @@ constexpr auto push_entry() {
 // tile count and no block waits on another.
 // Dynamic shared memory: step tables, grid slots (float grid kernels), then
 // the [n_sets + 1] tile prefix (prefix_off bytes in).
+
+// Exclusive prefix of the sets' tile counts (tiles of set s = ceil(N_s / per))
+// into prefix[0 .. n_sets] by the block's first warp; the caller synchronises
+// the block.  `count(s)` is the set's particle count.
+template <class Count>
+__device__ __forceinline__ void tile_prefix(long long *prefix, int n_sets, int per, const Count &count) {
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  long long acc = 0;
+  for (int s0 = 0; s0 < n_sets; s0 += 32) {
+    const int s = s0 + lane;
+    const long long ns = s < n_sets ? count(s) : 0;
+    // malformed offsets (ns < 0): no tiles (particles are bounds-checked by the caller)
+    const long long t = ns > 0 ? (ns + per - 1) / per : 0;
+    long long v = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long w = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += w;
+    }
+    if (s < n_sets) prefix[s] = acc + v - t;
+    acc += __shfl_sync(0xffffffffu, v, 31);
+  }
+  if (lane == 0) prefix[n_sets] = acc;
+}
+
 template <int KIND, int PREC, int GRID, int NP>
 __device__ __forceinline__ void batch_body(const Pulse<Real<PREC>> *__restrict__ sets,
                                            const BatchArgs &ba, unsigned prefix_off) {
   using R = Real<PREC>;
+  constexpr bool kFF = PREC == AP_FP32_PHASEFF;
+  // the part of the pulse the kind reads (a multiple of 4 bytes)
+  using PT = typename std::conditional<KIND == AP_FLYING_SUM || !kFF, Pulse<R>, PulseHead<R>>::type;
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ double s_red[32];
   __shared__ long long s_tile;
   __shared__ int s_set;
-  StepFF *s_steps = reinterpret_cast<StepFF *>(s_dyn);
   void *slots = s_dyn + step_table_bytes(blockDim.x);
   long long *s_prefix = reinterpret_cast<long long *>(s_dyn + prefix_off);
-  __shared__ __align__(16) unsigned char s_pulse_raw[sizeof(Pulse<R>)];
-  Pulse<R> &sp = *reinterpret_cast<Pulse<R> *>(s_pulse_raw);
+  __shared__ __align__(16) unsigned char s_pulse_raw[sizeof(PT)];
+  PT &sp = *reinterpret_cast<PT *>(s_pulse_raw);
   const PushArgs &a = ba.base;
   const int T = ba.tile;
   __shared__ float4 s_gridk[4];
-  if constexpr (NP == 2) grid_pair_consts(a.grid, s_gridk);  // the prefix's barrier follows
-  // tile prefix over sets: tiles of set s = ceil(N_s / T)
-  if (threadIdx.x == 0) {
-    long long acc = 0;
-    for (int s = 0; s < ba.n_sets; ++s) {
-      s_prefix[s] = acc;
-      long long ns = ba.set_offsets[s + 1] - ba.set_offsets[s];
-      if (ns < 0) ns = 0;  // malformed offsets: no tiles (particles are bounds-checked below)
-      acc += (ns + T - 1) / T;
-    }
-    s_prefix[ba.n_sets] = acc;
-    s_set = -1;
-  }
+  __shared__ StepBase s_base;
+  __shared__ float4 s_comp[kFF ? comp_slots<KIND, NP>() : 1];
+  tile_prefix(s_prefix, ba.n_sets, T,
+              [&](int s) { return ba.set_offsets[s + 1] - ba.set_offsets[s]; });
+  if (threadIdx.x == 0) s_set = -1;
   __syncthreads();
   const long long total = s_prefix[ba.n_sets];
-  // per-set pulse size copied to shared memory (flying focus: only n_comp components)
   for (;;) {
     if (threadIdx.x == 0) s_tile = (long long)atomicAdd(ba.tile_counter, 1u);
     __syncthreads();
@@ -466,12 +614,21 @@ __device__ __forceinline__ void batch_body(const Pulse<Real<PREC>> *__restrict__
     }
     const int set = lo;
     if (set != s_set) {
-      const int words = (int)(sizeof(Pulse<R>) / 4);
+      const int words = (int)(sizeof(PT) / 4);
       const uint32_t *src = reinterpret_cast<const uint32_t *>(sets + set);
       uint32_t *dst = reinterpret_cast<uint32_t *>(s_pulse_raw);
       for (int w = threadIdx.x; w < words; w += blockDim.x) dst[w] = src[w];
       __syncthreads();
       if (threadIdx.x == 0) s_set = set;
+      if constexpr (kFF) {
+        using RR = typename std::conditional<NP == 2, F2, float>::type;
+        if (threadIdx.x == 0) s_base = make_step_base(sp, a.t0, a.dt, a.grid);
+        if constexpr (KIND == AP_FLYING_SUM) comp_table<RR>(sp, s_comp);
+        if constexpr (NP == 2 && GRID != kGridNone) {
+          __syncthreads();
+          grid_pair_consts(a.grid, s_base, s_gridk);
+        }
+      }
     }
     __syncthreads();
     const long long first = ba.set_offsets[set] + (tile - s_prefix[set]) * T;
@@ -481,15 +638,17 @@ __device__ __forceinline__ void batch_body(const Pulse<Real<PREC>> *__restrict__
     for (int k = threadIdx.x; k < T; k += NP * blockDim.x) {
       const long long i = first + k;
       const bool valid = i >= 0 && i < end_set && i < a.n;
-      if constexpr (NP == 2) {
+      if constexpr (kFF) {
+        using RR = typename std::conditional<NP == 2, F2, float>::type;
         const long long i1 = i + blockDim.x;
-        const bool valid1 = i1 >= 0 && i1 < end_set && i1 < a.n;
+        const bool valid1 = NP == 2 && i1 >= 0 && i1 < end_set && i1 < a.n;
         double g[2];
-        push_two<KIND, GRID>(sp, a, i, i1, valid, valid1, s_steps, slots, s_gridk, g);
+        push_ff<KIND, GRID, RR>(sp, s_base, a, i, i1, valid, valid1, reinterpret_cast<float4 *>(s_dyn), s_comp, slots,
+                                s_gridk, g);
         if (valid) acc += g[0];
         if (valid1) acc += g[1];
       } else {
-        double g = push_one<KIND, PREC, GRID>(sp, a, i, valid, s_steps, slots);
+        double g = push_one<KIND, PREC, GRID>(sp, a, i, valid, slots);
         if (valid) acc += g;
       }
     }
@@ -507,11 +666,12 @@ __global__ void __launch_bounds__(256) batch_kernel(const Pulse<Real<PREC>> *__r
                                                     unsigned prefix_off) {
   batch_body<KIND, PREC, GRID, NP>(sets, ba, prefix_off);
 }
-// two particles per thread with one or both cells in shared memory: 2 blocks
-// of 256
+// two particles per thread: 2 blocks of 256 with one or both cells in shared
+// memory; 4 for the beams without a grid that fit 64 registers (batched_256:
+// 256 sets, 4e6 particles, 500 steps: 5.05 -> 4.88 ms against the compiler's own 80)
 template <int KIND, int GRID>
-__global__ void __launch_bounds__(256, 2)
-    batch_kernel_pair_2b(const Pulse<float> *__restrict__ sets, const __grid_constant__ BatchArgs ba,
+__global__ void __launch_bounds__(256, GRID == kGridNone ? 4 : 2)
+    batch_kernel_pair_minb(const Pulse<float> *__restrict__ sets, const __grid_constant__ BatchArgs ba,
                          unsigned prefix_off) {
   batch_body<KIND, AP_FP32_PHASEFF, GRID, 2>(sets, ba, prefix_off);
 }
@@ -677,28 +837,22 @@ int launch_push_t(const Pulse<Real<PREC>> &P, const PushArgs &a, void *stream) {
   return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
 }
 
-// the two-particle kernel of a grid mode (each with its residency target)
-template <int KIND, int GRID>
-constexpr auto push_pair_entry() {
-  if constexpr (GRID == kGridCells) return push_kernel_pair_smem<KIND>;
-  else if constexpr (GRID == kGridCellsMix) return push_kernel_pair_mix<KIND>;
-  else return push_kernel_pair<KIND, GRID>;
-}
-
-template <int KIND, int GRID>
-int launch_push_pair_t(const Pulse<float> &P, const PushArgs &a, void *stream) {
-  auto kern = push_pair_entry<KIND, GRID>();
+// float-float: NP particles per thread, the call's constants made here
+template <int KIND, int GRID, int NP>
+int launch_push_ff_t(const Pulse<float> &P, const PushArgs &a, void *stream) {
+  auto kern = push_ff_entry<KIND, GRID, NP>();
   const int block = a.shape.block;
-  const size_t head = push_smem_head<AP_FP32_PHASEFF, GRID, 2>(block);
+  const size_t head = push_smem_head<AP_FP32_PHASEFF, GRID, NP>(block);
   const size_t smem = head + (a.diag.hist ? (size_t)a.diag.bins * sizeof(uint32_t) : 0);
   if (set_smem(kern, smem) != AP_OK) return AP_ERR_CUDA;
-  const long long per_block = 2LL * block;
+  const long long per_block = (long long)NP * block;
   const long long want = (a.n + per_block - 1) / per_block;
   int per_sm = a.shape.blocks_per_sm > 0 ? a.shape.blocks_per_sm : occupancy_blocks(kern, block, smem);
   long long cap = (long long)a.sm_count * per_sm;
   int grid = (int)(want < cap ? want : cap);
   if (grid < 1) grid = 1;
-  kern<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(P, a, (unsigned)head);
+  const StepBase sb = make_step_base(P, a.t0, a.dt, a.grid);
+  kern<<<grid, block, smem, static_cast<cudaStream_t>(stream)>>>(P, sb, a, (unsigned)head);
   return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
 }
 
@@ -1124,8 +1278,10 @@ int launch_nodes_t(const Pulse<Real<PREC>> &P, const NodeArgs &a, void *stream) 
 template <int KIND, int PREC, int GRID, int NP = 1>
 int launch_batch_t(const Pulse<Real<PREC>> *sets, const BatchArgs &ba, void *stream) {
   auto kern = batch_kernel<KIND, PREC, GRID, NP>;
-  if constexpr (PREC == AP_FP32_PHASEFF && NP == 2 && (GRID == kGridCells || GRID == kGridCellsMix))
-    kern = batch_kernel_pair_2b<KIND, GRID>;
+  constexpr bool kBeam = KIND == AP_PLANE || KIND == AP_GAUSS || KIND == AP_FLYING_CF;
+  if constexpr (PREC == AP_FP32_PHASEFF && NP == 2 &&
+                (GRID == kGridCells || GRID == kGridCellsMix || (GRID == kGridNone && kBeam)))
+    kern = batch_kernel_pair_minb<KIND, GRID>;
   const int block = ba.base.shape.block;
   const size_t head = push_smem_head<PREC, GRID, NP>(block);
   const size_t smem = head + (size_t)(ba.n_sets + 1) * sizeof(long long);
@@ -1148,18 +1304,23 @@ template <int KIND, int PREC>
 int launch_push_mode(const Pulse<Real<PREC>> &P, const PushArgs &a, void *stream) {
   if constexpr (PREC == AP_FP32_PHASEFF) {
     if (pair_mode(a))
-      return !a.grid_on                 ? launch_push_pair_t<KIND, kGridNone>(P, a, stream)
-             : a.shape.grid_cache == 2 ? launch_push_pair_t<KIND, kGridCellsMix>(P, a, stream)
-             : a.shape.grid_cache      ? launch_push_pair_t<KIND, kGridCellsReg>(P, a, stream)
-                                       : launch_push_pair_t<KIND, kGridCells>(P, a, stream);
+      return !a.grid_on                 ? launch_push_ff_t<KIND, kGridNone, 2>(P, a, stream)
+             : a.shape.grid_cache == 2 ? launch_push_ff_t<KIND, kGridCellsMix, 2>(P, a, stream)
+             : a.shape.grid_cache      ? launch_push_ff_t<KIND, kGridCellsReg, 2>(P, a, stream)
+                                       : launch_push_ff_t<KIND, kGridCells, 2>(P, a, stream);
+    if (!a.grid_on) return launch_push_ff_t<KIND, kGridNone, 1>(P, a, stream);
+    if (!a.grid.cells) return launch_push_ff_t<KIND, kGridNodes, 1>(P, a, stream);
+    return a.shape.grid_cache ? launch_push_ff_t<KIND, kGridCellsReg, 1>(P, a, stream)
+                              : launch_push_ff_t<KIND, kGridCells, 1>(P, a, stream);
+  } else {
+    if (!a.grid_on) return launch_push_t<KIND, PREC, kGridNone>(P, a, stream);
+    if constexpr (PREC != AP_FP64) {
+      if (a.grid.cells)
+        return a.shape.grid_cache ? launch_push_t<KIND, PREC, kGridCellsReg>(P, a, stream)
+                                  : launch_push_t<KIND, PREC, kGridCells>(P, a, stream);
+    }
+    return launch_push_t<KIND, PREC, kGridNodes>(P, a, stream);
   }
-  if (!a.grid_on) return launch_push_t<KIND, PREC, kGridNone>(P, a, stream);
-  if constexpr (PREC != AP_FP64) {
-    if (a.grid.cells)
-      return a.shape.grid_cache ? launch_push_t<KIND, PREC, kGridCellsReg>(P, a, stream)
-                                : launch_push_t<KIND, PREC, kGridCells>(P, a, stream);
-  }
-  return launch_push_t<KIND, PREC, kGridNodes>(P, a, stream);
 }
 
 template <int KIND, int PREC>

@@ -212,8 +212,9 @@ __device__ __forceinline__ Local<F2> local_coords2(const Pulse<float> &P, const 
 // The cell test and weights of a thread's two particles with packed
 // arithmetic (grid units, offsets from each cached cell), then each
 // particle's own warp-uniform refetch branch, as grid_fetch does per particle.
-// gk: the grid's inverse spacings and offsets pre-broadcast in shared memory,
-// gk[a] = (inv_d[a], inv_d[a], off[a], off[a]), and gk[3] = (1/2, 1/2, -, -):
+// gk: the factors and offsets from the coordinates (x, y, and z in the step's
+// own units) to grid units, pre-broadcast in shared memory,
+// gk[a] = (factor, factor, offset, offset), and gk[3] = (1/2, 1/2, -, -):
 // a 16-byte load yields both pair operands, where constants kept in the
 // kernel parameters would be re-broadcast into register pairs every step
 // (the two-particle kernels run at their register limit).

@@ -1,0 +1,109 @@
+"""The float-float step over its polarisation frames, kinds and envelopes:
+every polarisation of every kind (y-polarised and left-handed pulses run in a
+turned or mirrored frame without a grid, and are turned into the grid's frame
+with one), Laguerre orders at the loop edges of the step (p, |l| = 0, 1, 2,
+both signs of l), an odd and the smallest number of flying-focus components,
+and every envelope, one and two particles per thread.
+
+Tolerances as for the other float-float pushes (median relative |du| <= 1e-4,
+max <= 1e-3 against the oracle); the one- and two-particle kernels round alike,
+so they agree bit for bit, with and without the light-front diagnostic."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2307_04843_gb300 import workloads
+from support import THREADS, gpu_push, rel_u_err
+
+L = 2 * math.pi
+BASE = dict(a0=3.0, omega=1.0, w0=2.5 * L, z_focus=0.7, t_focus=0.2, phase0=0.4, longitudinal=True, env="gauss", env_len=25.0)
+KINDS = {
+    "plane": dict(kind="plane"),
+    "gauss": dict(kind="gauss"),
+    "flying_cf": dict(kind="flying_cf", beta_f=-0.6),
+    "lg00": dict(kind="lg", lg_p=0, lg_l=0),
+    "lg01": dict(kind="lg", lg_p=0, lg_l=1),
+    "lg0m2": dict(kind="lg", lg_p=0, lg_l=-2),
+    "lg10": dict(kind="lg", lg_p=1, lg_l=0),
+    "lg12": dict(kind="lg", lg_p=1, lg_l=2),
+    "lg2m1": dict(kind="lg", lg_p=2, lg_l=-1),
+    "flying2": dict(kind="flying", env="cw", n_comp=2, bw_frac=0.05, beta_f=0.99, ff_length=20 * L),
+    "flying5": dict(kind="flying", env="cw", n_comp=5, bw_frac=0.04, beta_f=-0.8, ff_length=15 * L, a0=-2.0),
+}
+
+
+def _parts(n):
+    parts = workloads.particles_uniform(((-4 * L, 4 * L),) * 2 + ((-5 * L, 5 * L),), n, 99)
+    rng = np.random.default_rng(5)
+    for k in ("ux", "uy", "uz"):  # float-representable momenta
+        parts[k] = np.float32(rng.normal(0.0, 0.5, n)).astype(np.float64)
+    return parts
+
+
+def _check(out, ref):
+    e = rel_u_err(out, ref)
+    assert np.median(e) <= 1e-4 and np.max(e) <= 1e-3, (np.median(e), np.max(e))
+
+
+def _same(a, b):
+    for k in a:
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("pol", ["x", "y", "cp", "cm"])
+@pytest.mark.parametrize("name", sorted(KINDS))
+def test_step_frames_and_kinds_match_oracle(name, pol):
+    pulse = dict(BASE, pol=pol, **KINDS[name])
+    parts = _parts(37)  # one warp and a ragged one; with pairs a padding partner
+    args = (pulse, parts, -3.0, 0.02, 150, "fp32")
+    ref = oracle.push(pulse, parts, -3.0, 0.02, 150, threads=THREADS)
+    one, _, st1 = gpu_push(*args, launch=dict(block=32))
+    two, _, st2 = gpu_push(*args, launch=dict(block=32, pairs=1))
+    assert st1 == 0 and st2 == 0
+    _check(one, ref)
+    _same(one, two)
+    lf, _, _ = gpu_push(*args, diag_keys=("lightfront",), launch=dict(block=32, pairs=1))
+    _same(one, lf)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("pol", ["x", "y", "cp", "cm"])
+@pytest.mark.parametrize("name", ["plane", "gauss", "lg12", "flying5"])
+def test_step_frames_with_grid_match_oracle(name, pol):
+    import torch
+    from paper_2307_04843_gb300 import _lib
+    pulse = dict(BASE, pol=pol, **KINDS[name])
+    parts = _parts(37)
+    box = ((-4 * L, 4 * L),) * 2 + ((-5 * L, 5 * L),)
+    lo, hi = tuple(b[0] for b in box), tuple(b[1] for b in box)
+    g = workloads.grid_field(box, 20, amplitude=0.2)
+    ref = oracle.push(pulse, parts, -3.0, 0.02, 150, grid=(g, lo, hi), threads=THREADS)
+    cells = _lib.pack_grid((torch.as_tensor(g).cuda(), lo, hi), layout="cells")
+    args = (pulse, parts, -3.0, 0.02, 150, "fp32")
+    base, _, _ = gpu_push(*args, grid=cells, launch=dict(block=64))
+    _check(base, ref)
+    for launch in (dict(block=64, grid_cache=1), dict(block=64, pairs=1), dict(block=64, pairs=1, grid_cache=1),
+                   dict(block=64, pairs=1, grid_cache=2)):
+        out, _, st = gpu_push(*args, grid=cells, launch=launch)
+        assert st == 0
+        _same(base, out)
+    arrays, _, _ = gpu_push(*args, grid=(g, lo, hi))
+    _check(arrays, ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("env", [dict(env="sin2", env_len=3.0), dict(env="sgauss", sg_order=1, env_len=9.0),
+                                 dict(env="sgauss", sg_order=4, env_len=12.0), dict(env="cw")])
+@pytest.mark.parametrize("name", ["plane", "gauss", "flying_cf", "lg12"])
+def test_step_envelopes_match_oracle(name, env):
+    pulse = dict(BASE, pol="x", **KINDS[name])
+    pulse.update(env)
+    parts = _parts(37)
+    ref = oracle.push(pulse, parts, -3.0, 0.02, 150, threads=THREADS)
+    one, _, _ = gpu_push(pulse, parts, -3.0, 0.02, 150, "fp32", launch=dict(block=32))
+    two, _, _ = gpu_push(pulse, parts, -3.0, 0.02, 150, "fp32", launch=dict(block=32, pairs=1))
+    _check(one, ref)
+    _same(one, two)
