@@ -35,6 +35,7 @@ namespace apt {
 constexpr int kAdjBlock = 128;
 constexpr int kAdjBlocksPerSm = 4;
 constexpr int kAdjMaxK = 256;
+constexpr int kAdjSlotsPerSm = 768;    // particle slots of the workspace
 constexpr int kAdjStateBytes = 48;  // one saved state: 6 doubles or 9 floats
 // tangents: x, y, z - z_f, w0 and, for the closed-form flying focus only,
 // beta_f (the other kinds do not depend on it: a fifth tangent would be
@@ -525,17 +526,9 @@ __global__ void __launch_bounds__(kAdjBlock, (PREC == AP_FP64 || GRID) ? 2 : kAd
   Pulse<R> &P = *reinterpret_cast<Pulse<R> *>(s_pulse_raw);
   const PushArgs &a = aa.base;
   const int Tt = blockDim.x;
-  if (threadIdx.x == 0) {
-    long long acc = 0;
-    for (int s = 0; s < aa.n_sets; ++s) {
-      s_prefix[s] = acc;
-      long long ns = aa.set_offsets ? aa.set_offsets[s + 1] - aa.set_offsets[s] : a.n;
-      if (ns < 0) ns = 0;
-      acc += (ns + Tt - 1) / Tt;
-    }
-    s_prefix[aa.n_sets] = acc;
-    s_set = -1;
-  }
+  tile_prefix(s_prefix, aa.n_sets, Tt,
+              [&](int s) { return aa.set_offsets ? aa.set_offsets[s + 1] - aa.set_offsets[s] : a.n; });
+  if (threadIdx.x == 0) s_set = -1;
   __syncthreads();
   const long long total = s_prefix[aa.n_sets];
   const size_t slot = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -679,41 +672,225 @@ __global__ void __launch_bounds__(kAdjBlock, (PREC == AP_FP64 || GRID) ? 2 : kAd
 
 // ------------------------------------------------- two particles per thread
 // The float-float adjoint of the Gaussian kinds without a grid, with each
-// thread carrying two particles in the two halves of packed (f32x2) values,
-// as the two-particle push does: the forward sweep, the recomputation, the
-// closed-form field derivatives and the Boris reverse all run on pairs.  Tiles
-// hold 2 kAdjBlock particles of one set (thread t: t and t + kAdjBlock).
-// Checkpoints and the tape keep the layout of the one-particle kernel with
-// the two particles of a thread side by side: [..][W][thread slots] float2,
-// the same bytes for half as many thread slots.
-constexpr int kAdjPairBlocksPerSm = 3;  // 156-162 registers, no spills
+// thread carrying two particles in the two halves of packed (f32x2) values.
+// The forward sweep and the recomputation are the steps of the push
+// (ap_step.cuh), in the pulse's frame; the reverse step is written for them.
+// Tiles hold 2 kAdjBlock particles of one set (thread t: t and t + kAdjBlock).
+//
+// Bound by the FP32 pipe and its dependency chains: 155 operations per
+// particle-step in the two forward passes and about 155 in the reverse step,
+// where differentiating the field in each direction and the generic Boris
+// reverse took 307 (and the two forward passes 250).  Measured, 64 sets, 1e6
+// particles, 200 steps: 3.9 -> 2.47 ms with 3 blocks per SM (144 registers,
+// FMA pipe 58 %, 12 warps) -> 2.30 ms with 4 (128 registers, 16 B spilled).
+constexpr int kAdjPairBlocksPerSm = 4;
 
+// A checkpoint holds the whole state; a tape entry what the reverse step
+// reads (x and y to float, Z and the momentum).
 struct PairIO {
-  static constexpr int W = 9;
-  __device__ static void put(float2 *b, size_t s, const Pos2 &p, const F2 u[3]) {
-    b[0 * s] = make_float2(p.x.hi.x, p.x.hi.y); b[1 * s] = make_float2(p.x.lo.x, p.x.lo.y);
-    b[2 * s] = make_float2(p.y.hi.x, p.y.hi.y); b[3 * s] = make_float2(p.y.lo.x, p.y.lo.y);
-    b[4 * s] = make_float2(p.dz.hi.x, p.dz.hi.y); b[5 * s] = make_float2(p.dz.lo.x, p.dz.lo.y);
-    b[6 * s] = make_float2(u[0].x, u[0].y); b[7 * s] = make_float2(u[1].x, u[1].y);
-    b[8 * s] = make_float2(u[2].x, u[2].y);
+  static constexpr int kCkpt = 9, kTape = 7;
+  template <bool FULL>
+  __device__ __forceinline__ static void put(float2 *b, size_t s, const FF2 &x, const FF2 &y, const FF2 &z, const F2 u[3]) {
+    b[0 * s] = f2v(x.hi); b[1 * s] = f2v(y.hi); b[2 * s] = f2v(z.hi); b[3 * s] = f2v(z.lo);
+    b[4 * s] = f2v(u[0]); b[5 * s] = f2v(u[1]); b[6 * s] = f2v(u[2]);
+    if constexpr (FULL) { b[7 * s] = f2v(x.lo); b[8 * s] = f2v(y.lo); }
   }
-  __device__ static void get(const float2 *b, size_t s, Pos2 &p, F2 u[3]) {
-    float2 v;
-    v = b[0 * s]; p.x.hi = F2(v.x, v.y); v = b[1 * s]; p.x.lo = F2(v.x, v.y);
-    v = b[2 * s]; p.y.hi = F2(v.x, v.y); v = b[3 * s]; p.y.lo = F2(v.x, v.y);
-    v = b[4 * s]; p.dz.hi = F2(v.x, v.y); v = b[5 * s]; p.dz.lo = F2(v.x, v.y);
-    v = b[6 * s]; u[0] = F2(v.x, v.y); v = b[7 * s]; u[1] = F2(v.x, v.y);
-    v = b[8 * s]; u[2] = F2(v.x, v.y);
+  template <bool FULL>
+  __device__ __forceinline__ static void get(const float2 *b, size_t s, FF2 &x, FF2 &y, FF2 &z, F2 u[3]) {
+    x.hi = pair::f2of(b[0 * s]); y.hi = pair::f2of(b[1 * s]); z.hi = pair::f2of(b[2 * s]); z.lo = pair::f2of(b[3 * s]);
+    u[0] = pair::f2of(b[4 * s]); u[1] = pair::f2of(b[5 * s]); u[2] = pair::f2of(b[6 * s]);
+    if constexpr (FULL) { x.lo = pair::f2of(b[7 * s]); y.lo = pair::f2of(b[8 * s]); }
   }
 };
 
-// reverse_step for a thread's two particles (Gaussian kinds, no grid)
-template <int KIND>
-__device__ __forceinline__ void reverse_step_pair(const Pulse<float> &P, float dt, const StepFF &st,
-                                                  const Pos2 &pos, const F2 u[3], F2 lx[3], F2 lu[3],
-                                                  F2 g[kNp]) {
-  const Local<F2> L = local_coords2(P, st, pos);
-  beam_reverse<KIND == AP_FLYING_CF>(P, L, F2(P.a0), u, F2(dt), F2(P.adv_xy), lx, lu, g, NoGridPart{});
+// The reverse step's own constants: the factors of StepBase for a unit
+// amplitude, and those of the field's derivatives with the amplitude in.
+struct RevConst {
+  float hbr, hce, hcb;    // h times B0/E0, the E_z and the B_z factor
+  float dxy, dt;          // position increments per unit velocity
+  float w2, zr, k, eta;   // 2/w0^2, 1/z_R, k, and 2 ln2 s_env / v_g, times a0
+  float a0, vg;           // a0; a0 / v_g (envelopes other than the Gaussian)
+  float zr1, omb;         // 1/z_R and 1/(1 - beta_f)
+};
+
+// Gamma'/Gamma of the envelope at eta s_env (see envelope_dlog), times 1: the
+// general form, for envelopes other than the Gaussian
+template <class PT>
+__device__ __forceinline__ F2 dlog_scaled(const PT &P, F2 e, F2 mul) {
+  switch (P.env) {
+    case AP_ENV_SIN2: {
+      F2 s, c;
+      sincos_r(e, &s, &c);
+      return unless_zero(F2(-2.0f * P.fast.s_env) * s * rcp_r(c), mul);
+    }
+    case AP_ENV_GAUSS:
+      return F2(-1.38629436f * P.fast.s_env) * e;
+    case AP_ENV_SGAUSS: {
+      const F2 s = e * e;
+      F2 p = F2(1.0f);
+      for (int i = 1; i < P.sg_order; ++i) p *= s;
+      return F2(-1.38629436f * P.env_b * (float)P.sg_order * P.fast.s_env) * e * p;
+    }
+    default:
+      return F2(0.0f);
+  }
+}
+
+// One reverse step for a thread's two particles: state (x, y, Z, u) before the
+// step, adjoints lx (of x, y, z - z_f), lu after it, updated to before it.
+//
+// With q = 1/(1 - i zeta), a = r^2/w0^2, M the unit-amplitude envelope and
+// carrier times e^{-a q}: U = q M, W = q U, and the unit fields are Re U, Im U,
+// and x, y times Re W, Im W.  Let c be the cotangent of the fields (from the
+// Boris reverse) in complex form, so that F . dF = Re(cU dU) + Re(cW dW) +
+// (terms of x and y themselves).  Every derivative of U and W is a factor
+// times U and W,
+//   dU = U alpha, dW = W (alpha + i q dzeta),
+//   alpha = i q (1 - a q) dzeta - q da + (Gamma'/Gamma) deta + i dpsi,
+// so with Y = cU U + cW W the derivatives in da, dzeta, deta, dpsi are the
+// four real numbers
+//   S_a = -Re(q Y), S_zeta = Re(i q (1 - a q) Y) + Re(i q cW W),
+//   (Gamma'/Gamma) Re Y, -Im Y,
+// formed once, and each direction (x, y, z - z_f, w0, beta_f) is a short real
+// combination of them.  Re Y is also F . f, the derivative in a0.
+// gr: d/da0, -(w0/2) d/dw0 / a0, d/dz_f, d/dbeta_f / a0.
+template <int KIND, int POL, int ENV, class PT>
+__device__ __forceinline__ void reverse_step_pair(const PT &P, const StepBase &sb, const RevConst &rc, const float4 st,
+                                                  F2 x, F2 y, F2 zhi, F2 zlo, const F2 u[3], F2 lx[3], F2 lu[3],
+                                                  F2 gr[kNp]) {
+  using R = F2;
+  const FastPulse &F = P.fast;
+  // unit fields, as in unit_fields_beam
+  const R eta = rfma(zhi, R(F.c_eta), R(st.y));
+  R mul, g;
+  envelope_fast<ENV>(P, eta, mul, g);
+  const R zn = KIND == AP_FLYING_CF ? rfma(zhi, R(F.c_zn), R(st.z)) : rmul(zhi, R(F.c_zn));
+  const R inv = rcp_r(rfma(zn, zn, R(1.0f)));
+  const R nq = rmul(zn, inv), qi = rneg(nq);
+  const R b = rmul(rfma(x, x, rmul(y, y)), R(F.c_a));
+  const R ang = phase_angle(rfma(b, rmul(nq, R(kTurnsPerExp)), R(st.x)), zhi, zlo);
+  R sn, cs;
+  sincos_r(ang, &sn, &cs);
+  R mag = exp2_neg(rfma(b, inv, g));
+  if constexpr (ENV == kEnvAny) mag = rmul(mag, mul);
+  const R mc = rmul(mag, cs), ms = rmul(mag, sn);
+  const R Ur = rfma(inv, mc, rmul(nq, ms)), Ui = rfma(inv, ms, rmul(qi, mc));
+  const R Wr = rfma(inv, Ur, rmul(nq, Ui)), Wi = rfma(inv, Ui, rmul(qi, Ur));
+  const R ny = rneg(y);
+  const R ez = POL == kLin ? rmul(x, Wi) : rfma(x, Wi, rmul(ny, Wr));
+  const R bz = POL == kLin ? rmul(y, Wi) : rfma(x, Wr, rmul(y, Wi));
+  // Boris forward intermediates (boris_unit)
+  const R a0 = rfma(R(sb.hA), Ur, u[0]), a1 = POL == kCirc ? rfma(R(sb.hA), Ui, u[1]) : u[1];
+  const R a2 = rfma(R(sb.hAce), ez, u[2]);
+  const R am[3] = {a0, a1, a2};
+  const R ig = inv_gamma(am);
+  const R hb = rmul(R(sb.hAbr), ig);
+  const R t1 = rmul(hb, Ur), nt1 = rneg(t1);
+  const R t2 = rmul(rmul(R(sb.hAcb), ig), bz), nt2 = rneg(t2);
+  R t0 = R(0.0f), nt0 = R(0.0f);
+  R tt = rfma(t1, t1, rfma(t2, t2, R(1.0f)));
+  R p0 = rfma(a1, t2, rfma(a2, nt1, a0)), p1 = rfma(a0, nt2, a1), p2 = rfma(a0, t1, a2);
+  if constexpr (POL == kCirc) {
+    nt0 = rmul(hb, Ui);
+    t0 = rneg(nt0);
+    tt = rfma(t0, t0, tt);
+    p1 = rfma(a2, t0, p1);
+    p2 = rfma(a1, nt0, p2);
+  }
+  const R ii = rcp_r(tt);
+  const R f = radd(ii, ii);
+  const R s1 = rmul(f, t1), s2 = rmul(f, t2), ns1 = rneg(s1), ns2 = rneg(s2);
+  const R s0 = POL == kCirc ? rmul(f, t0) : R(0.0f), ns0 = POL == kCirc ? rneg(s0) : R(0.0f);
+  R un[3] = {rfma(R(sb.hA), Ur, rfma(p1, s2, rfma(p2, ns1, a0))), rfma(p0, ns2, a1), rfma(p0, s1, a2)};
+  if constexpr (POL == kCirc) {
+    un[1] = rfma(R(sb.hA), Ui, rfma(p2, s0, un[1]));
+    un[2] = rfma(p1, ns0, un[2]);
+  }
+  un[2] = rfma(R(sb.hAce), ez, un[2]);
+  const R ign = inv_gamma(un);
+  // position update: ub = lu + (d - v (v . d)) / gamma', d = dt lx
+  const R v[3] = {rmul(un[0], ign), rmul(un[1], ign), rmul(un[2], ign)};
+  const R d[3] = {rmul(R(rc.dxy), lx[0]), rmul(R(rc.dxy), lx[1]), rmul(R(rc.dt), lx[2])};
+  const R nvl = rneg(rfma(v[0], d[0], rfma(v[1], d[1], rmul(v[2], d[2]))));
+  const R b0 = rfma(ign, rfma(v[0], nvl, d[0]), lu[0]), b1 = rfma(ign, rfma(v[1], nvl, d[1]), lu[1]);
+  const R b2 = rfma(ign, rfma(v[2], nvl, d[2]), lu[2]);
+  // rotation: pb = s x ub, sbar = ub x p, ab = ub + pb + t x pb, tb = pb x a + ds/dt sbar
+  R pb0 = rfma(s1, b2, rmul(ns2, b1)), pb1 = rmul(s2, b0), pb2 = rmul(ns1, b0);
+  if constexpr (POL == kCirc) {
+    pb1 = rfma(ns0, b2, pb1);
+    pb2 = rfma(s0, b1, pb2);
+  }
+  const R nb0 = rneg(b0), npb0 = rneg(pb0);
+  const R sb1 = rfma(b2, p0, rmul(nb0, p2)), sb2 = rfma(b0, p1, rmul(rneg(b1), p0));
+  R ab0 = rfma(t1, pb2, rfma(nt2, pb1, radd(b0, pb0)));
+  R ab1 = rfma(t2, pb0, radd(b1, pb1));
+  R ab2 = rfma(t1, npb0, radd(b2, pb2));
+  R tb1 = rfma(pb2, a0, rmul(npb0, a2)), tb2 = rfma(pb0, a1, rmul(rneg(pb1), a0));
+  R ts = rfma(t1, sb1, rmul(t2, sb2));
+  R tb0 = R(0.0f);
+  R sb0 = R(0.0f);
+  if constexpr (POL == kCirc) {
+    ab1 = rfma(nt0, pb2, ab1);
+    ab2 = rfma(t0, pb1, ab2);
+    sb0 = rfma(b1, p2, rmul(rneg(b2), p1));
+    tb0 = rfma(pb1, a2, rmul(rneg(pb2), a1));
+    ts = rfma(t0, sb0, ts);
+  }
+  // s = f t, f = 2/(1 + t^2): tb += f (sbar - f (t . sbar) t)
+  const R nfts = rneg(rmul(f, ts));
+  tb1 = rfma(f, rfma(nfts, t1, sb1), tb1);
+  tb2 = rfma(f, rfma(nfts, t2, sb2), tb2);
+  if constexpr (POL == kCirc) tb0 = rfma(f, rfma(nfts, t0, sb0), tb0);
+  // t = h B / gamma: the cotangent of 1/gamma is (t . tb) gamma
+  R tt2 = rfma(t1, tb1, rmul(t2, tb2));
+  if constexpr (POL == kCirc) tt2 = rfma(t0, tb0, tt2);
+  const R c3 = rneg(rmul(rmul(ig, ig), tt2));
+  ab0 = rfma(c3, a0, ab0);
+  ab1 = rfma(c3, a1, ab1);
+  ab2 = rfma(c3, a2, ab2);
+  lu[0] = ab0;
+  lu[1] = ab1;
+  lu[2] = ab2;
+  // cotangents of the unit fields' parts
+  const R hb1 = rmul(R(rc.hbr), ig);
+  const R cR = rfma(R(sb.h), radd(b0, ab0), rmul(hb1, tb1));
+  const R cE = rmul(R(rc.hce), radd(b2, ab2)), cB = rmul(rmul(R(rc.hcb), ig), tb2);
+  const R cWi = rfma(cE, x, rmul(cB, y));
+  R Zr = rmul(cWi, Wi), Zi = rmul(rneg(cWi), Wr);  // cW W
+  R Yr = rmul(cR, Ur), Yi = rmul(cR, Ui);
+  if constexpr (POL == kCirc) {
+    const R cWr = rfma(cB, x, rmul(cE, ny));
+    Zr = rfma(cWr, Wr, Zr);
+    Zi = rfma(cWr, Wi, Zi);
+    const R cI = rfma(R(sb.h), radd(b1, ab1), rmul(rneg(hb1), tb0));
+    Yr = rfma(cI, Ui, Yr);
+    Yi = rfma(rneg(cI), Ur, Yi);
+  }
+  Yr = radd(Yr, Zr);
+  Yi = radd(Yi, Zi);
+  const R Pr = rfma(inv, Yr, rmul(nq, Yi)), Pi = rfma(inv, Yi, rmul(qi, Yr));
+  const R qPi = rfma(inv, Pi, rmul(qi, Pr));
+  const R a = rmul(b, R(0.693147181f));
+  // S_zeta = a Im(q^2 Y) - Im(q Y) - Im(q cW W)
+  const R Sz = rsub(rfma(a, qPi, rmul(nq, Zr)), rfma(inv, Zi, Pi));
+  // direct terms of x and y, and the directions
+  const R wE = rmul(R(rc.a0), cE), wB = rmul(R(rc.a0), cB);
+  const R sa = rmul(R(-rc.w2), Pr);
+  lx[0] = rfma(sa, x, rfma(wE, Wi, lx[0]));
+  lx[1] = rfma(sa, y, rfma(wB, Wi, lx[1]));
+  if constexpr (POL == kCirc) {
+    lx[0] = rfma(wB, Wr, lx[0]);
+    lx[1] = rfma(rneg(wE), Wr, lx[1]);
+  }
+  R dz = rfma(R(rc.k), Yi, rmul(R(rc.zr), Sz));
+  if constexpr (ENV == kEnvGauss) dz = rfma(rmul(R(rc.eta), eta), Yr, dz);
+  else dz = rfma(rmul(R(-rc.vg), dlog_scaled(P, eta, mul)), Yr, dz);
+  lx[2] = radd(lx[2], dz);
+  gr[0] = radd(gr[0], Yr);
+  gr[1] = rfma(Pr, a, rfma(Sz, zn, rsub(gr[1], Zr)));
+  gr[2] = rsub(gr[2], dz);
+  if constexpr (KIND == AP_FLYING_CF)
+    gr[3] = rfma(Sz, rfma(zn, R(-rc.omb), R(-rc.zr1 * st.w)), gr[3]);
 }
 
 template <int KIND>
@@ -723,30 +900,25 @@ __global__ void __launch_bounds__(kAdjBlock, kAdjPairBlocksPerSm)
   __shared__ long long s_tile;
   __shared__ int s_set;
   __shared__ double s_red[32];
-  __shared__ StepFF s_steps[kAdjMaxK];
-  __shared__ __align__(16) unsigned char s_pulse_raw[sizeof(Pulse<float>)];
-  __shared__ long long s_prefix[AP_MAX_SETS + 1];
-  // dynamic: the next reverse step's tape entry, [2][W][kAdjBlock] float2
+  __shared__ float4 s_steps[kAdjMaxK];
+  __shared__ StepBase s_base;
+  __shared__ RevConst s_rev;
+  __shared__ __align__(16) unsigned char s_pulse_raw[sizeof(PulseHead<float>)];
+  // dynamic: the next reverse step's tape entry, [2][kTape][kAdjBlock] float2,
+  // then the [n_sets + 1] tile prefix
   extern __shared__ __align__(16) unsigned char s_adj_dyn[];
   float2 *s_next = reinterpret_cast<float2 *>(s_adj_dyn);
-  Pulse<float> &P = *reinterpret_cast<Pulse<float> *>(s_pulse_raw);
+  long long *s_prefix = reinterpret_cast<long long *>(s_adj_dyn + 2 * PairIO::kTape * kAdjBlock * sizeof(float2));
+  PulseHead<float> &P = *reinterpret_cast<PulseHead<float> *>(s_pulse_raw);
   const PushArgs &a = aa.base;
   constexpr int kPer = 2 * kAdjBlock;  // particles per tile
-  if (threadIdx.x == 0) {
-    long long acc = 0;
-    for (int s = 0; s < aa.n_sets; ++s) {
-      s_prefix[s] = acc;
-      long long ns = aa.set_offsets ? aa.set_offsets[s + 1] - aa.set_offsets[s] : a.n;
-      if (ns < 0) ns = 0;
-      acc += (ns + kPer - 1) / kPer;
-    }
-    s_prefix[aa.n_sets] = acc;
-    s_set = -1;
-  }
+  tile_prefix(s_prefix, aa.n_sets, kPer,
+              [&](int s) { return aa.set_offsets ? aa.set_offsets[s + 1] - aa.set_offsets[s] : a.n; });
+  if (threadIdx.x == 0) s_set = -1;
   __syncthreads();
   const long long total = s_prefix[aa.n_sets];
   const size_t slot = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t stride = (size_t)(aa.nslots / 2);  // thread slots
+  const size_t stride = (size_t)gridDim.x * kAdjBlock;  // thread slots
   float2 *ck = static_cast<float2 *>(aa.ckpt) + slot;
   float2 *tp = static_cast<float2 *>(aa.tape) + slot;
   const float *uxs = static_cast<const float *>(a.ux);
@@ -764,12 +936,20 @@ __global__ void __launch_bounds__(kAdjBlock, kAdjPairBlocksPerSm)
     }
     const int set = lo;
     if (set != s_set) {
-      const int words = (int)(sizeof(Pulse<float>) / 4);
+      const int words = (int)(sizeof(PulseHead<float>) / 4);
       const uint32_t *src = reinterpret_cast<const uint32_t *>(sets + set);
       uint32_t *dst = reinterpret_cast<uint32_t *>(s_pulse_raw);
       for (int w = threadIdx.x; w < words; w += blockDim.x) dst[w] = src[w];
       __syncthreads();
-      if (threadIdx.x == 0) s_set = set;
+      if (threadIdx.x == 0) {
+        s_set = set;
+        s_base = make_step_base(P, a.t0, a.dt, a.grid);
+        const float g = P.lon ? -2.0f * P.inv_w0sq : 0.0f, a0 = P.a0, h = s_base.h;
+        s_rev = RevConst{h * P.bratio, h * P.lonE * g, h * P.bratio * P.lonB * g,
+                         (float)a.dt * P.adv_xy, (float)a.dt,
+                         2.0f * P.inv_w0sq * a0, P.inv_zR * a0, (float)P.k * a0,
+                         1.38629436f * P.fast.s_env * P.inv_vg * a0, a0, P.inv_vg * a0, P.inv_zR, P.inv_1mb};
+      }
     }
     __syncthreads();
     const long long off0 = aa.set_offsets ? aa.set_offsets[set] : 0;
@@ -779,91 +959,111 @@ __global__ void __launch_bounds__(kAdjBlock, kAdjPairBlocksPerSm)
     const bool v0 = i0 >= 0 && i0 < off1 && i0 < a.n;
     const bool v1 = i1 >= 0 && i1 < off1 && i1 < a.n;
     const double Ns = (double)(off1 - off0);
-    // ---- forward pass with checkpoints
-    double X[2] = {0.0, 0.0}, Y[2] = {0.0, 0.0}, Z[2] = {0.0, 0.0};
-    float ua[3] = {0.0f, 0.0f, 0.0f}, ub[3] = {0.0f, 0.0f, 0.0f};
-    if (v0) {
-      X[0] = a.x[i0]; Y[0] = a.y[i0]; Z[0] = a.z[i0];
-      ua[0] = uxs[i0]; ua[1] = uys[i0]; ua[2] = uzs[i0];
-    }
-    if (v1) {
-      X[1] = a.x[i1]; Y[1] = a.y[i1]; Z[1] = a.z[i1];
-      ub[0] = uxs[i1]; ub[1] = uys[i1]; ub[2] = uzs[i1];
-    }
-    Pos2 pos;
-    pos.load(X, Y, Z, P.z_f);
-    F2 u[3] = {F2(ua[0], ub[0]), F2(ua[1], ub[1]), F2(ua[2], ub[2])};
-    TimeBase<AP_FP32_PHASEFF> tb;
-    tb.init(P, a.t0, a.dt);
-    const float dts = (float)a.dt;
-    const F2 dtR = dts, dtxy = dts * P.adv_xy;
-    for (int seg = 0; seg < aa.n_seg; ++seg) {
-      const long long s0 = (long long)seg * aa.K;
-      const int cnt = (int)(a.n_steps - s0 < aa.K ? a.n_steps - s0 : aa.K);
-      PairIO::put(ck + (size_t)seg * PairIO::W * stride, stride, pos, u);
-      __syncthreads();
-      for (int k = threadIdx.x; k < cnt; k += blockDim.x) s_steps[k] = tb.at(s0 + k);
-      __syncthreads();
-      for (int k = 0; k < cnt; ++k) {
-        const Local<F2> L = local_coords2(P, s_steps[k], pos);
-        F2 E[3], B[3];
-        analytic_fields<KIND, AP_FP32_PHASEFF, F2>(P, L, E, B);
-        const F2 ig = boris(u, E, B, dtR);
-        pos.advance(u[0] * ig, u[1] * ig, u[2] * ig, dtxy, dtR);
-      }
-    }
-    // ---- objective and seed, per particle
-    const float uf[2][3] = {{u[0].x, u[1].x, u[2].x}, {u[0].y, u[1].y, u[2].y}};
-    double gN[2], Jv = 0.0;
-    float sd[2][3];
-    for (int h = 0; h < 2; ++h) {
-      const bool vh = h ? v1 : v0;
-      gN[h] = sqrt(1.0 + (double)uf[h][0] * uf[h][0] + (double)uf[h][1] * uf[h][1] +
-                   (double)uf[h][2] * uf[h][2]);
-      for (int k = 0; k < 3; ++k) sd[h][k] = vh ? (float)((double)uf[h][k] / (gN[h] * Ns)) : 0.0f;
-      if (vh) Jv += gN[h] / Ns;
-    }
-    F2 lx[3] = {F2(0.0f), F2(0.0f), F2(0.0f)};
-    F2 lu[3] = {F2(sd[0][0], sd[1][0]), F2(sd[0][1], sd[1][1]), F2(sd[0][2], sd[1][2])};
-    double gacc[kNp] = {0.0, 0.0, 0.0, 0.0};
-    // ---- reverse sweep over segments
-    for (int seg = aa.n_seg - 1; seg >= 0; --seg) {
-      const long long s0 = (long long)seg * aa.K;
-      const int cnt = (int)(a.n_steps - s0 < aa.K ? a.n_steps - s0 : aa.K);
-      PairIO::get(ck + (size_t)seg * PairIO::W * stride, stride, pos, u);
-      __syncthreads();
-      for (int k = threadIdx.x; k < cnt; k += blockDim.x) s_steps[k] = tb.at(s0 + k);
-      __syncthreads();
-      for (int k = 0; k < cnt; ++k) {
-        PairIO::put(tp + (size_t)k * PairIO::W * stride, stride, pos, u);
-        const Local<F2> L = local_coords2(P, s_steps[k], pos);
-        F2 E[3], B[3];
-        analytic_fields<KIND, AP_FP32_PHASEFF, F2>(P, L, E, B);
-        const F2 ig = boris(u, E, B, dtR);
-        pos.advance(u[0] * ig, u[1] * ig, u[2] * ig, dtxy, dtR);
-      }
-      // the tape entries this thread just stored are read back by its own
-      // asynchronous copies
-      __threadfence_block();
-      auto stage = [&](int k) {
-        const float2 *src = tp + (size_t)k * PairIO::W * stride;
+    // ---- load, in the pulse's frame
+    FF px[2], py[2], pz[2];
+    float uu[2][3];
 #pragma unroll
-        for (int w = 0; w < PairIO::W; ++w)
-          cp_async8((unsigned)__cvta_generic_to_shared(s_next + ((k & 1) * PairIO::W + w) * kAdjBlock +
-                                                       threadIdx.x),
-                    src + (size_t)w * stride);
-      };
-      F2 gs[kNp] = {F2(0.0f), F2(0.0f), F2(0.0f), F2(0.0f)};
-      stage(cnt - 1);
-      for (int k = cnt - 1; k >= 0; --k) {
-        cp_async_wait_all();
-        PairIO::get(s_next + (k & 1) * PairIO::W * kAdjBlock + threadIdx.x, kAdjBlock, pos, u);
-        if (k > 0) stage(k - 1);
-        reverse_step_pair<KIND>(P, dts, s_steps[k], pos, u, lx, lu, gs);
+    for (int h = 0; h < 2; ++h) {
+      px[h] = py[h] = pz[h] = FF{0.0f, 0.0f};
+      uu[h][0] = uu[h][1] = uu[h][2] = 0.0f;
+      if (h ? v1 : v0) {
+        const long long i = h ? i1 : i0;
+        px[h] = split_double(a.x[i]);
+        py[h] = split_double(a.y[i]);
+        pz[h] = split_double(__dmul_rn(__dsub_rn(a.z[i], P.z_f), P.fast.z_scale));
+        uu[h][0] = uxs[i];
+        uu[h][1] = uys[i];
+        uu[h][2] = uzs[i];
+        to_frame(P.fast.frame, px[h], py[h], uu[h]);
       }
-      for (int k = 0; k < kNp; ++k)
-        gacc[k] += (v0 ? (double)gs[k].x : 0.0) + (v1 ? (double)gs[k].y : 0.0);
     }
+    FF2 x{F2(px[0].hi, px[1].hi), F2(px[0].lo, px[1].lo)};
+    FF2 y{F2(py[0].hi, py[1].hi), F2(py[0].lo, py[1].lo)};
+    FF2 z{F2(pz[0].hi, pz[1].hi), F2(pz[0].lo, pz[1].lo)};
+    F2 u[3] = {F2(uu[0][0], uu[1][0]), F2(uu[0][1], uu[1][1]), F2(uu[0][2], uu[1][2])};
+    double Jv = 0.0, gacc[kNp] = {0.0, 0.0, 0.0, 0.0};
+
+    auto sweep = [&](auto pol_c, auto env_c) {
+      constexpr int POL = decltype(pol_c)::value, ENV = decltype(env_c)::value;
+      auto table = [&](long long s0, int cnt) {
+        __syncthreads();
+        for (int k = threadIdx.x; k < cnt; k += blockDim.x)
+          s_steps[k] = step_entry<KIND>(P.fast, s_base, (float)(int)(s0 + k));
+        __syncthreads();
+      };
+      auto step = [&](int k) {
+        const UnitFields<F2> f = unit_fields<KIND, POL, ENV>(P, nullptr, s_steps[k], x.hi, y.hi, z.hi, z.lo);
+        const F2 ig = boris_unit<POL, true>(u, f, s_base);
+        const F2 kxy = rmul(F2(s_base.cxy), ig);
+        advance(x, u[0], kxy);
+        advance(y, u[1], kxy);
+        advance(z, u[2], rmul(F2(s_base.cz), ig));
+      };
+      // ---- forward pass with checkpoints
+      for (int seg = 0; seg < aa.n_seg; ++seg) {
+        const long long s0 = (long long)seg * aa.K;
+        const int cnt = (int)(a.n_steps - s0 < aa.K ? a.n_steps - s0 : aa.K);
+        PairIO::put<true>(ck + (size_t)seg * PairIO::kCkpt * stride, stride, x, y, z, u);
+        table(s0, cnt);
+        for (int k = 0; k < cnt; ++k) step(k);
+      }
+      // ---- objective and seed, per particle
+      float sd[2][3];
+      for (int h = 0; h < 2; ++h) {
+        const bool vh = h ? v1 : v0;
+        const double d0 = lane_of(u[0], h), d1 = lane_of(u[1], h), d2 = lane_of(u[2], h);
+        const double gN = sqrt(1.0 + d0 * d0 + d1 * d1 + d2 * d2);
+        const double w = vh ? 1.0 / (gN * Ns) : 0.0;
+        sd[h][0] = (float)(d0 * w);
+        sd[h][1] = (float)(d1 * w);
+        sd[h][2] = (float)(d2 * w);
+        if (vh) Jv += gN / Ns;
+      }
+      F2 lx[3] = {F2(0.0f), F2(0.0f), F2(0.0f)};
+      F2 lu[3] = {F2(sd[0][0], sd[1][0]), F2(sd[0][1], sd[1][1]), F2(sd[0][2], sd[1][2])};
+      // ---- reverse sweep over segments
+      for (int seg = aa.n_seg - 1; seg >= 0; --seg) {
+        const long long s0 = (long long)seg * aa.K;
+        const int cnt = (int)(a.n_steps - s0 < aa.K ? a.n_steps - s0 : aa.K);
+        PairIO::get<true>(ck + (size_t)seg * PairIO::kCkpt * stride, stride, x, y, z, u);
+        table(s0, cnt);
+        for (int k = 0; k < cnt; ++k) {
+          PairIO::put<false>(tp + (size_t)k * PairIO::kTape * stride, stride, x, y, z, u);
+          step(k);
+        }
+        // the tape entries this thread just stored are read back by its own
+        // asynchronous copies
+        __threadfence_block();
+        auto stage = [&](int k) {
+          const float2 *src = tp + (size_t)k * PairIO::kTape * stride;
+#pragma unroll
+          for (int w = 0; w < PairIO::kTape; ++w)
+            cp_async8((unsigned)__cvta_generic_to_shared(s_next + ((k & 1) * PairIO::kTape + w) * kAdjBlock +
+                                                         threadIdx.x),
+                      src + (size_t)w * stride);
+        };
+        F2 gs[kNp] = {F2(0.0f), F2(0.0f), F2(0.0f), F2(0.0f)};
+        stage(cnt - 1);
+        for (int k = cnt - 1; k >= 0; --k) {
+          cp_async_wait_all();
+          PairIO::get<false>(s_next + (k & 1) * PairIO::kTape * kAdjBlock + threadIdx.x, kAdjBlock, x, y, z, u);
+          if (k > 0) stage(k - 1);
+          reverse_step_pair<KIND, POL, ENV>(P, s_base, s_rev, s_steps[k], x.hi, y.hi, z.hi, z.lo, u, lx, lu, gs);
+        }
+        for (int k = 0; k < kNp; ++k)
+          gacc[k] += (v0 ? (double)gs[k].x : 0.0) + (v1 ? (double)gs[k].y : 0.0);
+      }
+    };
+    using Lin = std::integral_constant<int, kLin>;
+    using Circ = std::integral_constant<int, kCirc>;
+    using EnvG = std::integral_constant<int, kEnvGauss>;
+    using EnvA = std::integral_constant<int, kEnvAny>;
+    if (P.fast.circ) sweep(Circ{}, EnvA{});
+    else if (P.env == AP_ENV_GAUSS) sweep(Lin{}, EnvG{});
+    else sweep(Lin{}, EnvA{});
+    gacc[1] *= 2.0 * (double)P.inv_w0 * (double)P.a0;
+    gacc[3] *= (double)P.a0;
+
     if ((v0 || v1) && !(isfinite(gacc[0]) && isfinite(gacc[1]) && isfinite(gacc[2]) && isfinite(gacc[3])))
       atomicOr(a.status, kStatusNonfinite);
     // per-set reduction (every particle of the tile belongs to `set`)
@@ -879,14 +1079,38 @@ __global__ void __launch_bounds__(kAdjBlock, kAdjPairBlocksPerSm)
   }
 }
 
+// The two-particle kernel's segment length: any split of the steps whose
+// checkpoints (9 floats) and tape (7 floats per step) fit the caller's
+// workspace (n_seg + K states of 12 floats for aa.nslots particles, shared out
+// over `slots` here) gives the same result, and the shorter the segment the
+// smaller the tape.  From 16 steps up it stays in the L2 cache (70 MB of 129 at
+// 16 steps; at 100 steps 436 MB would go through HBM, 56 bytes per
+// particle-step), below 16 the checkpoints' own traffic grows.
+inline void pair_segments(AdjArgs &aa, long long slots) {
+  const long long n = aa.base.n_steps, budget = 12LL * (aa.n_seg + aa.K) * aa.nslots / slots;
+  for (int K = 16; K < aa.K; K += 4) {
+    const long long seg = (n + K - 1) / K;
+    if (PairIO::kCkpt * seg + PairIO::kTape * K <= budget) {
+      aa.K = K;
+      aa.n_seg = (int)seg;
+      return;
+    }
+  }
+}
+
 template <int KIND>
-int launch_adjoint_pair(const Pulse<float> *sets, const AdjArgs &aa, void *stream) {
+int launch_adjoint_pair(const Pulse<float> *sets, const AdjArgs &a0, void *stream) {
   auto kern = adjoint_kernel_pair<KIND>;
-  const size_t dyn = 2 * (size_t)PairIO::W * kAdjBlock * sizeof(float2);
-  // static (about 40 KB) plus dynamic shared memory passes 48 KB: opt in
+  AdjArgs aa = a0;
+  const int grid = aa.base.sm_count * kAdjPairBlocksPerSm;
+  const long long slots = (long long)grid * 2 * kAdjBlock;
+  static_assert(kAdjPairBlocksPerSm * 2 * kAdjBlock * 3 <= kAdjSlotsPerSm * 4,
+                "9 n_seg + 7 K floats fit the workspace for every K");
+  pair_segments(aa, slots);
+  aa.tape = static_cast<char *>(aa.ckpt) + sizeof(float) * PairIO::kCkpt * (size_t)aa.n_seg * (size_t)slots;
+  const size_t dyn = 2 * (size_t)PairIO::kTape * kAdjBlock * sizeof(float2) + (size_t)(aa.n_sets + 1) * sizeof(long long);
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
     return AP_ERR_CUDA;
-  const int grid = (int)(aa.nslots / (2 * kAdjBlock));
   kern<<<grid, kAdjBlock, dyn, static_cast<cudaStream_t>(stream)>>>(sets, aa);
   return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
 }
@@ -930,13 +1154,10 @@ int handle_push_args(ap_handle h, const ap_particles *p, const ap_grid *g, doubl
 }  // namespace apt
 
 namespace {
-// particle slots of the workspace: the larger of the one-particle kernel's
-// (kAdjBlocksPerSm blocks of kAdjBlock per SM) and the two-particle
-// kernel's (kAdjPairBlocksPerSm blocks of 2 kAdjBlock particles)
-long long adj_slots(int sm_count) {
-  const int a = apt::kAdjBlocksPerSm * apt::kAdjBlock, b = apt::kAdjPairBlocksPerSm * 2 * apt::kAdjBlock;
-  return (long long)sm_count * (a > b ? a : b);
-}
+// particle slots of the workspace (the one-particle kernel uses kAdjBlocksPerSm
+// blocks of kAdjBlock per SM of them; the two-particle kernel shares the same
+// bytes out over its own slots)
+long long adj_slots(int sm_count) { return (long long)sm_count * apt::kAdjSlotsPerSm; }
 }  // namespace
 
 extern "C" {

@@ -233,6 +233,21 @@ __device__ __forceinline__ R pack_lanes(float a, float b) {
 __device__ __forceinline__ float lane_of(float v, int) { return v; }
 __device__ __forceinline__ float lane_of(F2 v, int h) { return h ? v.y : v.x; }
 
+// a state into the pulse's frame
+__device__ __forceinline__ void to_frame(int frame, FF &x, FF &y, float u[3]) {
+  if (frame == 1) {
+    const FF t = x;
+    x = y;
+    y = FF{-t.hi, -t.lo};
+    const float tu = u[0];
+    u[0] = u[1];
+    u[1] = -tu;
+  } else if (frame == 2) {
+    y = FF{-y.hi, -y.lo};
+    u[1] = -u[1];
+  }
+}
+
 template <int KIND, int GRID, typename R, class PT>
 __device__ __forceinline__ void push_ff(const PT &P, const StepBase &sb, const PushArgs &a, long long i0, long long i1,
                                         bool v0, bool v1, float4 *s_steps, const float4 *comps, void *slots,
@@ -257,17 +272,7 @@ __device__ __forceinline__ void push_ff(const PT &P, const StepBase &sb, const P
       uu[h][0] = static_cast<const float *>(a.ux)[i];
       uu[h][1] = static_cast<const float *>(a.uy)[i];
       uu[h][2] = static_cast<const float *>(a.uz)[i];
-      if (frame == 1) {
-        const FF t = px[h];
-        px[h] = py[h];
-        py[h] = FF{-t.hi, -t.lo};
-        const float tu = uu[h][0];
-        uu[h][0] = uu[h][1];
-        uu[h][1] = -tu;
-      } else if (frame == 2) {
-        py[h] = FF{-py[h].hi, -py[h].lo};
-        uu[h][1] = -uu[h][1];
-      }
+      to_frame(frame, px[h], py[h], uu[h]);
     }
     // light-front reference h0 = gamma - u_z on entry
     h0[h] = 1.0f / rsqrt_r(fmaf(uu[h][0], uu[h][0], fmaf(uu[h][1], uu[h][1], fmaf(uu[h][2], uu[h][2], 1.0f)))) -

@@ -156,8 +156,8 @@ __host__ __device__ inline StepBase make_step_base(const PulseHead<float> &P, do
 }
 
 // The step table's entry for step n (an integer below 2^23, in float):
-// {C_n in turns, |C_n| <= 1/2; then, by kind: T_n scaled for the envelope and
-// for the moving focus; or, for the flying-focus sum, T_n in turns as hi, lo}.
+// {C_n in turns, |C_n| <= 1/2; T_n scaled for the envelope, for the moving
+// focus, and itself}; for the flying-focus sum {-, -, T_n in turns as hi, lo}.
 template <int KIND>
 __device__ __forceinline__ float4 step_entry(const FastPulse &F, const StepBase &s, float nf) {
   const FF nt = two_prod(nf, s.DT.hi);
@@ -171,7 +171,7 @@ __device__ __forceinline__ float4 step_entry(const FastPulse &F, const StepBase 
     const float clo = __fadd_rn(__fadd_rn(c.lo, nd.lo), __fmaf_rn(nf, s.del.lo, s.om0.lo));
     const float C = __fadd_rn(__fsub_rn(c.hi, round_magic(c.hi)), clo);
     return make_float4(C, __fmaf_rn(T.hi, F.s_env, __fmul_rn(T.lo, F.s_env)),
-                       __fmaf_rn(T.hi, F.c_tz, __fmul_rn(T.lo, F.c_tz)), 0.0f);
+                       __fmaf_rn(T.hi, F.c_tz, __fmul_rn(T.lo, F.c_tz)), __fadd_rn(T.hi, T.lo));
   }
 }
 
