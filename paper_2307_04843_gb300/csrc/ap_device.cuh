@@ -297,7 +297,7 @@ struct Local {
 };
 
 template <int PREC>
-__device__ __forceinline__ Local<Real<PREC>> local_coords(const Pulse<Real<PREC>> &P,
+__device__ __forceinline__ Local<Real<PREC>> local_coords(const PulseHead<Real<PREC>> &P,
                                                           const typename TimeBase<PREC>::Step &st,
                                                           const Pos<PREC> &pos) {
   Local<Real<PREC>> L;

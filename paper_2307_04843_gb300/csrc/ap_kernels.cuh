@@ -1119,6 +1119,159 @@ __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_consta
   }
 }
 
+// Gaussian beams (AP_GAUSS, AP_FLYING_CF) in float-float arithmetic, three or
+// more components: exp(-(x^2 + y^2) q / w0^2) is a product of an x and a y
+// factor, so with z fixed every node value is
+//   v = Re(X P) + x Re(X Q),
+// X the complex x factor of the node's column and P, Q complex numbers of its
+// row (Q only for the longitudinal components).  A warp takes slabs of one z
+// index, 128 columns and up to 32 rows: each lane keeps the x factors of its
+// four columns (whole and half node, both z levels) in registers, lane l makes
+// the 16 coefficients of row l, and the rows then cost 18 FP32 operations per
+// node and no special functions.  The rows of all column blocks are divided
+// evenly over one resident wave of warps (a warp's share may span slabs).  Per-node evaluation took 122 instructions
+// and 18 special-function operations and was bound by latency at half the
+// store bandwidth; this is bound by the stores (256^3, 402 MB: 88.5 -> 72.6 us, 5.5 TB/s).  The
+// factors are made with the accurate library functions (each is used by tens of nodes), so that their
+// product is as good as one approximate exponential was.
+// VEC: four consecutive columns per lane and 16-byte accesses (rows aligned to
+// 16 bytes); otherwise columns 32 apart.
+constexpr int kSlabCols = 128;
+constexpr int kSlabRows = 32;  // at most; one lane makes one row's coefficients
+
+// e^{-a q} with a >= 0 a real number times 1/w0^2: 2^-(a log2e Re q), angle -a Im q
+__device__ __forceinline__ Cx<float> beam_factor(float a, Cx<float> q, float turn) {
+  const float mag = exp2f(-(a * q.re) * (float)kLog2e);
+  float s, c;
+  // the angle in half turns, reduced by sincospif
+  sincospif(2.0f * fmaf(-a * q.im, kInvTwoPi, turn), &s, &c);
+  return {mag * c, mag * s};
+}
+
+template <int KIND, typename T, bool VEC>
+__global__ void __launch_bounds__(256) nodes_slab_kernel(const __grid_constant__ PulseHead<float> P,
+                                                         const __grid_constant__ NodeArgs a) {
+  using W = typename std::conditional<(sizeof(T) > sizeof(float)), T, float>::type;
+  __shared__ float4 s_row[8][kSlabRows][4];
+  unsigned want = 0u;
+  for (int q = 0; q < a.n_comp; ++q) want |= 1u << a.comp[q];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nxc = (a.nx + kSlabCols - 1) / kSlabCols;
+  const long long total = (long long)nxc * a.nz * a.ny;  // rows of column blocks, (k, block, j) in order
+  const long long n_warps = (long long)gridDim.x * 8, wid = (long long)blockIdx.x * 8 + warp;
+  const long long per = total / n_warps, more = total - per * n_warps;
+  long long row = wid * per + (wid < more ? wid : more);
+  const long long row_end = row + per + (wid < more ? 1 : 0);
+  TimeBase<AP_FP32_PHASEFF> tb;
+  tb.init(P, a.t, 0.0);
+  const StepFF st = tb.at(0);
+  constexpr int kStep = VEC ? 1 : 32;
+  long long kb_cur = -1;
+  int k = 0, i0 = 0;
+  Cx<float> q[2];            // of the two z levels
+  float amp[2], turn[2];     // envelope and carrier
+  float xw[4];
+  Cx<float> X[2][2][4];      // x factors of the lane's columns: [z level][whole, half]
+  while (row < row_end) {
+    const long long kb = row / a.ny;
+    const int j0 = (int)(row - kb * a.ny);
+    int nj = a.ny - j0 < kSlabRows ? a.ny - j0 : kSlabRows;
+    if (nj > row_end - row) nj = (int)(row_end - row);
+    row += nj;
+    if (kb != kb_cur) {
+      kb_cur = kb;
+      k = (int)(kb / nxc);
+      i0 = (int)(kb - (long long)k * nxc) * kSlabCols + (VEC ? 4 * lane : lane);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        Pos<AP_FP32_PHASEFF> pos;
+        pos.x = FF{0.0f, 0.0f};
+        pos.y = FF{0.0f, 0.0f};
+        pos.z = node_coord_ff((float)k + (h ? 0.5f : 0.0f), a.lo_hi[2], a.lo_lo[2], a.d_hi[2], a.d_lo[2]);
+        const BeamZ<float> b = gauss_z<KIND == AP_FLYING_CF>(P, local_coords<AP_FP32_PHASEFF>(P, st, pos));
+        q[h] = b.q;
+        amp[h] = b.amp_mul * exp2f(b.l2);
+        turn[h] = b.psi * kInvTwoPi;
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const float fi = (float)(i0 + m * kStep);
+        xw[m] = fmaf(fi, a.d_hi[0], a.lo_hi[0]);
+        const float xh = fmaf(fi + 0.5f, a.d_hi[0], a.lo_hi[0]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          X[h][0][m] = beam_factor(xw[m] * xw[m] * P.inv_w0sq, q[h], 0.0f);
+          X[h][1][m] = beam_factor(xh * xh * P.inv_w0sq, q[h], 0.0f);
+        }
+      }
+    }
+    // row coefficients of row j0 + lane
+    if (lane < nj) {
+      const float fj = (float)(j0 + lane);
+      const float y[2] = {fmaf(fj, a.d_hi[1], a.lo_hi[1]), fmaf(fj + 0.5f, a.d_hi[1], a.lo_hi[1])};
+      auto row = [&](int h, int o) {  // U less its x factor
+        const Cx<float> f = beam_factor(y[o] * y[o] * P.inv_w0sq, q[h], turn[h]);
+        return cscale(cmul(q[h], f), amp[h]);
+      };
+      const float g = -2.0f * P.inv_w0sq, ce = P.lon ? P.lonE * g : 0.0f, cb = P.lon ? P.bratio * P.lonB * g : 0.0f;
+      const float br = P.bratio;
+      const Cx<float> u00 = row(0, 0), u01 = row(0, 1), u10 = row(1, 0), u11 = row(1, 1);
+      const Cx<float> wz = cmul(q[1], u10), wb = cmul(q[0], u01);  // W of Ez and of Bz
+      // E = Re[p U], B_perp = br Re[(z x p) U]; E_z = ce Im[(p_x x + p_y y) W],
+      // B_z = cb Im[(p_x y - p_y x) W]; Im w = Re(-i w)
+      const Cx<float> px{P.px_re, P.px_im}, py{P.py_re, P.py_im};
+      auto mi = [](Cx<float> w, float s) { return Cx<float>{s * w.im, -s * w.re}; };
+      const Cx<float> p0 = cmul(px, u00), p1 = cmul(py, u01), p3 = cscale(cmul(py, u11), -br), p4 = cscale(cmul(px, u10), br);
+      const Cx<float> q2 = mi(cmul(px, wz), ce), p2 = mi(cmul(py, wz), ce * y[0]);
+      const Cx<float> q5 = mi(cmul(py, wb), -cb), p5 = mi(cmul(px, wb), cb * y[1]);
+      float4 *r = s_row[warp][lane];
+      r[0] = make_float4(p0.re, p0.im, p1.re, p1.im);
+      r[1] = make_float4(p2.re, p2.im, q2.re, q2.im);
+      r[2] = make_float4(p3.re, p3.im, p4.re, p4.im);
+      r[3] = make_float4(p5.re, p5.im, q5.re, q5.im);
+    }
+    __syncwarp();
+    long long at = ((long long)k * a.ny + j0) * a.nx + i0;
+    for (int r = 0; r < nj; ++r, at += a.nx) {
+      const float4 c0 = s_row[warp][r][0], c1 = s_row[warp][r][1], c2 = s_row[warp][r][2], c3 = s_row[warp][r][3];
+      float v[6][4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        auto re = [](Cx<float> x, float cr, float ci) { return fmaf(x.re, cr, -(x.im * ci)); };
+        const Cx<float> w0 = X[0][0][m], h0 = X[0][1][m], w1 = X[1][0][m], h1 = X[1][1][m];
+        const float xh = fmaf((float)(i0 + m * kStep) + 0.5f, a.d_hi[0], a.lo_hi[0]);
+        v[0][m] = re(h0, c0.x, c0.y);
+        v[1][m] = re(w0, c0.z, c0.w);
+        v[2][m] = fmaf(xw[m], re(w1, c1.z, c1.w), re(w1, c1.x, c1.y));
+        v[3][m] = re(w1, c2.x, c2.y);
+        v[4][m] = re(h1, c2.z, c2.w);
+        v[5][m] = fmaf(xh, re(h0, c3.z, c3.w), re(h0, c3.x, c3.y));
+      }
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        if (!((want >> c) & 1u)) continue;
+        T *f = static_cast<T *>(a.f[c]) + at;
+        if constexpr (VEC) {
+          if (i0 < a.nx) {
+            float4 *f4 = reinterpret_cast<float4 *>(f);
+            float4 o = make_float4(v[c][0], v[c][1], v[c][2], v[c][3]);
+            if (a.accumulate) {
+              const float4 p = *f4;
+              o = make_float4(p.x + o.x, p.y + o.y, p.z + o.z, p.w + o.w);
+            }
+            *f4 = o;
+          }
+        } else {
+#pragma unroll
+          for (int m = 0; m < 4; ++m)
+            if (i0 + 32 * m < a.nx) f[32 * m] = a.accumulate ? (T)((W)f[32 * m] + (W)v[c][m]) : (T)v[c][m];
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // One warp writes the value v along a row of n elements (store, or add to
 // what the row holds, rounding once to T): a scalar head up to the first
 // 16-byte boundary, then 16-byte vector stores, then a scalar tail.  The row
@@ -1159,11 +1312,11 @@ __device__ __forceinline__ void row_put(T *__restrict__ row, int n, W v, bool ac
 
 // Plane waves (Eqs. plane_func, plane_b) depend on z and t only.  A row of
 // nx nodes (fixed y, z) holds two z positions: the whole node z_k (Ex, Ey,
-// Bz) and the half node z_k + dz/2 (Ez, Bx, By).  One warp per row
-// evaluates the field once at each position it needs (every lane computes
-// the same value), then streams each requested component along its row with
-// 16-byte stores, so for nx >= 32 the kernel is bound by the stores, not the
-// arithmetic.
+// Bz) and the half node z_k + dz/2 (Ez, Bx, By).  Each warp takes a contiguous
+// run of rows and evaluates the field once per z index at each position it
+// needs (every lane computes the same value), then streams each requested
+// component along its rows with 16-byte stores, so for nx >= 32 the kernel is
+// bound by the stores, not the arithmetic.
 template <int PREC, typename T>
 __global__ void __launch_bounds__(256) nodes_plane_kernel(const __grid_constant__ Pulse<Real<PREC>> P,
                                                           const __grid_constant__ NodeArgs a) {
@@ -1181,9 +1334,15 @@ __global__ void __launch_bounds__(256) nodes_plane_kernel(const __grid_constant_
   TimeBase<PREC> tb;
   tb.init(P, a.t, 0.0);
   const typename TimeBase<PREC>::Step st = tb.at(0);
-  for (long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += warps) {
+  const long long per = (rows + warps - 1) / warps;
+  const long long r0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
+  const long long r1 = r0 + per < rows ? r0 + per : rows;
+  int kcur = -1;
+  R v[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
+  for (long long r = r0; r < r1; ++r) {
     const int k = (int)(r / a.ny);
-    R v[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
+    if (k != kcur) {
+      kcur = k;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (!need[h]) continue;
@@ -1208,6 +1367,7 @@ __global__ void __launch_bounds__(256) nodes_plane_kernel(const __grid_constant_
         v[3] = B[0];
         v[4] = B[1];
       }
+    }
     }
     for (int i = 0; i < a.n_comp; ++i) {
       const int c = a.comp[i];
@@ -1243,7 +1403,19 @@ int launch_nodes_t(const Pulse<Real<PREC>> &P, const NodeArgs &a, void *stream) 
     if (gx < 1) gx = 1;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if constexpr (PREC == AP_FP32_PHASEFF && KIND != AP_PLANE) {
-      // beams in float-float arithmetic: two nodes per lane, packed; one
+      if constexpr (KIND == AP_GAUSS || KIND == AP_FLYING_CF) {
+        bool vec = !a.f64 && a.nx % 4 == 0;
+        for (int i = 0; i < a.n_comp; ++i) vec = vec && (reinterpret_cast<uintptr_t>(a.f[a.comp[i]]) & 15u) == 0;
+        auto kern = a.f64 ? nodes_slab_kernel<KIND, double, false>
+                    : vec ? nodes_slab_kernel<KIND, float, true> : nodes_slab_kernel<KIND, float, false>;
+        // one resident wave, and at least four rows for each warp's set-up
+        const long long units = (long long)((a.nx + kSlabCols - 1) / kSlabCols) * rows;
+        long long gp = (long long)a.sm_count * occupancy_blocks(kern, block, 0);
+        if (gp > (units + 31) / 32) gp = (units + 31) / 32;
+        kern<<<(unsigned)gp, block, 0, s>>>(P, a);
+        return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
+      }
+      // other beams in float-float arithmetic: two nodes per lane, packed; one
       // resident wave of blocks, each warp a contiguous run of rows
       if (!a.current) {
         auto kern = a.f64 ? nodes_row_pair_kernel<KIND, double> : nodes_row_pair_kernel<KIND, float>;
