@@ -182,6 +182,8 @@ struct LineArgs {
   float z0_hi, z0_lo, dz_hi, dz_lo;  // float-float node positions (AP_FP32_PHASEFF)
   long long n_steps;
 };
+constexpr int kPlasmaPairNodes = 8192;  // longest traditional float line in registers
+int launch_plasma_float(const LineArgs &a, void *stream);
 int launch_line(bool apt, int precision, const Pulse<double> &pd, const Pulse<float> &pf,
                 const LineArgs &a, void *stream);
 

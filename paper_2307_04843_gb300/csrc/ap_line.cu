@@ -11,8 +11,8 @@
 //     evaluated in the kernel every step (Eqs. E_1_j, E_2_j, j1).
 //
 // One block per line; the line (E, B, J and a_k = dt omega_p^2(z_k)) stays
-// on chip for all n_steps and is written back once: in registers for the
-// traditional float line up to 6144 nodes (plasma_line_reg_kernel), in
+// on chip for all n_steps and is written back once: in registers for float
+// lines of up to 8192 nodes (plasma_line_pair_kernel in ap_yee.cu, split_line_kernel), in
 // shared memory otherwise (line_kernel).  Per step of line_kernel: the
 // B half step; a barrier; the current and E update of each node (one pass:
 // both read only the node's own E and J and the neighbouring B); a barrier;
@@ -23,9 +23,12 @@
 // loop of the same expressions bit for bit.
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdint>
+#include <cstring>
 
 #include "ap_kernels.cuh"
+#include "ap_lines.cuh"
 
 namespace apt {
 namespace {
@@ -39,84 +42,25 @@ __device__ __forceinline__ float l_sub(float a, float b) { return __fsub_rn(a, b
 __device__ __forceinline__ float l_add(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float l_mul(float a, float b) { return __fmul_rn(a, b); }
 
-// Float-float split line: the node-dependent part of the carrier phase,
-// k (z_k - z_f) as float-float, and z_k - z_f, computed once per launch with
-// the operations of local_coords (so the phase and envelope argument of every
-// evaluation are those of the generic path bit for bit).
-struct NodeFF {
-  float kd_hi, kd_lo, dz;
-};
-
-__device__ __forceinline__ NodeFF node_ff(const Pulse<float> &P, const LineArgs &a, float fk) {
-  const FF z = node_coord_ff(fk, a.z0_hi, a.z0_lo, a.dz_hi, a.dz_lo);
-  FF dz = two_sum(z.hi, -P.zf_hi);
-  dz.lo = __fadd_rn(dz.lo, __fsub_rn(z.lo, P.zf_lo));
-  FF kd = two_prod(P.k_hi, dz.hi);
-  kd.lo = __fadd_rn(kd.lo, __fmaf_rn(P.k_hi, dz.lo, __fmul_rn(P.k_lo, dz.hi)));
-  return {kd.hi, kd.lo, __fadd_rn(dz.hi, dz.lo)};
-}
-
-// E1 at t_n and J1 at t_n + dt/2 at two nodes of the float split line at once
-// (the halves of every packed value, ap_pair.cuh: one issue slot per FP32
-// operation for both nodes, the MUFU operations one per node), for a plane
-// wave polarised along x (Eqs. plane_func, j1): the J1 carrier phase is the
-// E1 phase advanced by omega dt/2, applied as a fixed rotation (sin, cos of
-// omega dt/2 in sdl, cdl); the envelope and its log-derivatives are evaluated
-// at eta and eta + dt/2.
-__device__ __forceinline__ void line_sources_ff2(const Pulse<float> &P, const StepFF &st, F2 kd_hi, F2 kd_lo,
-                                                 F2 dz, float sdl, float cdl, float hdt, F2 &E1, F2 &J1) {
-  const FF2 ps = two_diff(F2(st.C), kd_hi);
-  const F2 psi = reduce_ff(ps.hi, ps.lo - kd_lo);
-  const float Tf = __fadd_rn(st.Th, st.Tl);
-  const F2 eta0 = fma(dz, F2(-P.inv_vg), F2(Tf));
-  F2 mul, l2;
-  envelope(P, eta0, mul, l2);
-  F2 a = F2(P.amp) * mul;
-  if (l2 != F2(0.0f)) a *= exp2_r(l2);  // exp2(0) = 1 exactly for a half without an exponent
-  F2 s, c;
-  sincos_r(psi, &s, &c);
-  E1 = a * c;
-  const F2 eta = eta0 + F2(hdt);
-  envelope(P, eta, mul, l2);
-  F2 aj = F2(P.jamp * P.amp) * mul;
-  if (l2 != F2(0.0f)) aj *= exp2_r(l2);
-  const F2 sj = fma(s, F2(cdl), c * F2(sdl)), cj = fma(s, F2(-sdl), c * F2(cdl));
-  F2 L1, L2;
-  envelope_logd(P, eta, L1, L2);
-  const Cx<F2> V = finite_duration(Cx<F2>{aj * cj, aj * sj}, 1.0f, L1, L2, P.inv_w);
-  J1 = V.im;  // Re[p (-i V)] with p = (1, 0)
-}
-
 // Local coordinates of node k (x = y = 0) at one time level (double).
-template <int PREC>
-__device__ __forceinline__ Local<Real<PREC>> node_local(const Pulse<Real<PREC>> &P, const LineArgs &a,
-                                                        const typename TimeBase<PREC>::Step &st, int k) {
-  Pos<PREC> pos;
-  if constexpr (PREC == AP_FP32_PHASEFF) {
-    pos.x = FF{0.0f, 0.0f};
-    pos.y = FF{0.0f, 0.0f};
-    pos.z = node_coord_ff((float)k, a.z0_hi, a.z0_lo, a.dz_hi, a.dz_lo);
-  } else {
-    pos.load(0.0, 0.0, __dadd_rn(a.z0, __dmul_rn((double)k, a.dz)));
-  }
-  return local_coords<PREC>(P, st, pos);
+__device__ __forceinline__ Local<double> node_local(const Pulse<double> &P, const LineArgs &a, double st, int k) {
+  Pos<AP_FP64> pos;
+  pos.load(0.0, 0.0, __dadd_rn(a.z0, __dmul_rn((double)k, a.dz)));
+  return local_coords<AP_FP64>(P, st, pos);
 }
 
-template <typename T, int PREC, bool APT>
-__global__ void __launch_bounds__(kLineBlock) line_kernel(const __grid_constant__ Pulse<Real<PREC>> P,
+// The line in shared memory: double lines, split (APT) or traditional, and
+// traditional float lines of more than 8192 nodes.
+template <typename T, bool APT>
+__global__ void __launch_bounds__(kLineBlock) line_kernel(const __grid_constant__ Pulse<double> P,
                                                           const __grid_constant__ LineArgs a) {
-  using R = Real<PREC>;
+  static_assert(!APT || sizeof(T) == 8, "the float split line runs in registers");
   extern __shared__ __align__(16) unsigned char line_smem[];
   const int nz = a.nz;
   T *e = reinterpret_cast<T *>(line_smem);
   T *b = e + nz;
   T *j = b + nz;
   T *q = j + nz;  // a_k = dt omega_p^2(z_k)
-  // float split line only: per-node phase constants (see NodeFF)
-  constexpr bool kFF = APT && PREC == AP_FP32_PHASEFF;
-  float *kdh = reinterpret_cast<float *>(q + nz);
-  float *kdl = kdh + nz;
-  float *dzn = kdl + nz;
   const size_t off = (size_t)blockIdx.x * (size_t)nz;
   T *Eg = static_cast<T *>(a.E) + off;
   T *Bg = static_cast<T *>(a.B) + off;
@@ -132,76 +76,36 @@ __global__ void __launch_bounds__(kLineBlock) line_kernel(const __grid_constant_
     b[k] = Bg[k];
     j[k] = Jg[k];
     q[k] = l_mul(dt, W ? W[k] : wpu);
-    if constexpr (kFF) {
-      const NodeFF c = node_ff(P, a, (float)k);
-      kdh[k] = c.kd_hi;
-      kdl[k] = c.kd_lo;
-      dzn[k] = c.dz;
-    }
   }
-  TimeBase<PREC> tb;
+  TimeBase<AP_FP64> tb;
   if constexpr (APT) tb.init(P, a.t0, 0.5 * a.dt);  // level 2n: t_n, 2n + 1: t_n + dt/2
-  float lev = 0.0f;  // 2n in float (exact: 2 n_steps + 1 < 2^24 is checked on the host)
-  float sdl = 0.0f, cdl = 1.0f;  // sin, cos of omega dt/2 (float split line)
-  if constexpr (kFF) {
-    double sd, cd;
-    sincos(0.5 * P.omega * a.dt, &sd, &cd);
-    sdl = (float)sd;
-    cdl = (float)cd;
-  }
-  const float hdt = (float)(0.5 * a.dt);
   __syncthreads();
   for (long long n = 0; n < a.n_steps; ++n) {
     // B^{n+1/2} = B^n - (r/2)(E_{k+1}^n - E_k^n)
     for (int k = t; k < nz - 1; k += bd) b[k] = l_sub(b[k], l_mul(hr, l_sub(e[k + 1], e[k])));
     __syncthreads();
-    typename TimeBase<PREC>::Step st_e{}, st_j{};
-    if constexpr (kFF) {
-      st_e = tb.at_f(lev);
-      lev += 2.0f;
-    } else if constexpr (APT) {
+    double st_e = 0.0, st_j = 0.0;
+    if constexpr (APT) {
       st_e = tb.at(2 * n);
       st_j = tb.at(2 * n + 1);
     }
     // J^{n+1/2} = J^{n-1/2} + a_k (E1 + E2)^n;  E^{n+1} = (E^n - r dB) - dt (J - J1)^{n+1/2}
-    if constexpr (kFF) {
-      // the thread's nodes k and k + bd in the two halves of one packed
-      // source evaluation; each node's update as below
-      auto update = [&](int k, float e1, float j1) {
-        const T ek = e[k];
-        const T jk = l_add(j[k], l_mul(q[k], l_add(e1, ek)));
-        j[k] = jk;
-        if (k >= 1) e[k] = l_sub(l_sub(ek, l_mul(r, l_sub(b[k], b[k - 1]))), l_mul(dt, l_sub(jk, j1)));
-      };
-      for (int k = t; k < nz; k += 2 * bd) {
-        const int k2 = k + bd;
-        const bool two = k2 < nz;
-        const int kk = two ? k2 : k;  // the second half repeats node k when k + bd is past the line
-        F2 e1, j1;
-        line_sources_ff2(P, st_e, F2(kdh[k], kdh[kk]), F2(kdl[k], kdl[kk]), F2(dzn[k], dzn[kk]), sdl, cdl, hdt,
-                         e1, j1);
-        update(k, e1.x, j1.x);
-        if (two) update(k2, e1.y, j1.y);
-      }
-    } else
     for (int k = t; k < nz; k += bd) {
       const T ek = e[k];
       T drive = ek;
       if constexpr (APT) {
-        R E1[3], B1[3];
-        const Local<R> L = node_local<PREC>(P, a, st_e, k);
-        analytic_fields<AP_PLANE, PREC>(P, L, E1, B1);
-        drive = l_add((T)E1[0], ek);
+        double E1[3], B1[3];
+        analytic_fields<AP_PLANE, AP_FP64>(P, node_local(P, a, st_e, k), E1, B1);
+        drive = l_add(E1[0], ek);
       }
       const T jk = l_add(j[k], l_mul(q[k], drive));
       j[k] = jk;
       if (k >= 1) {
         T src = jk;
         if constexpr (APT) {
-          R J1[3];
-          const Local<R> L = node_local<PREC>(P, a, st_j, k);
-          current_plane(P, L, J1);
-          src = l_sub(jk, (T)J1[0]);
+          double J1[3];
+          current_plane(P, node_local(P, a, st_j, k), J1);
+          src = l_sub(jk, J1[0]);
         }
         e[k] = l_sub(l_sub(ek, l_mul(r, l_sub(b[k], b[k - 1]))), l_mul(dt, src));
       }
@@ -218,96 +122,232 @@ __global__ void __launch_bounds__(kLineBlock) line_kernel(const __grid_constant_
   }
 }
 
-// Traditional line with the line in registers: thread t owns the C
-// consecutive nodes [t C, t C + C) of E, B, J and a_k; per step only the
-// values at thread boundaries move through shared memory, with two
-// barriers: (1) B half step (needs E at the next thread's first node, `en`),
-// publish the last B; barrier; (2) current and E update (needs B at the
-// previous thread's last node), publish the first E; barrier; (3) B half
-// step with the fresh `en`.  Each shared slot is written and read in
-// alternate barrier intervals.  The arithmetic per node is that of
-// line_kernel, so the result does not depend on C or the block size.
-template <typename T, int C, int MAXT>
-__global__ void __launch_bounds__(MAXT) plasma_line_reg_kernel(const __grid_constant__ LineArgs a) {
-  __shared__ T s_b[kLineBlock], s_e[kLineBlock];
-  const int nz = a.nz;
-  const size_t off = (size_t)blockIdx.x * (size_t)nz;
-  T *Eg = static_cast<T *>(a.E) + off;
-  T *Bg = static_cast<T *>(a.B) + off;
-  T *Jg = static_cast<T *>(a.J) + off;
-  const T *W = a.wp2 ? static_cast<const T *>(a.wp2) + off : nullptr;
-  const T dt = (T)a.dt;
-  const T r = (T)(a.dt / a.dz);
-  const T hr = (T)(0.5 * (a.dt / a.dz));
-  const T wpu = (T)a.omega_p2;
-  const int t = threadIdx.x;
-  const int base = t * C;
-  T e[C], b[C], j[C], q[C];
-#pragma unroll
-  for (int i = 0; i < C; ++i) {
-    const int k = base + i;
-    const bool in = k < nz;
-    e[i] = in ? Eg[k] : T(0);
-    b[i] = in ? Bg[k] : T(0);
-    j[i] = in ? Jg[k] : T(0);
-    q[i] = in ? l_mul(dt, W ? W[k] : wpu) : T(0);
-  }
-  s_e[t] = e[0];
-  __syncthreads();
-  T en = t + 1 < (int)blockDim.x ? s_e[t + 1] : T(0);
-  for (long long n = 0; n < a.n_steps; ++n) {
-#pragma unroll
-    for (int i = 0; i < C; ++i) {
-      const T enx = i + 1 < C ? e[i + 1] : en;
-      if (base + i < nz - 1) b[i] = l_sub(b[i], l_mul(hr, l_sub(enx, e[i])));
-    }
-    s_b[t] = b[C - 1];
-    __syncthreads();
-    const T bp = t > 0 ? s_b[t - 1] : T(0);
-#pragma unroll
-    for (int i = 0; i < C; ++i) {
-      const int k = base + i;
-      if (k < nz) {
-        j[i] = l_add(j[i], l_mul(q[i], e[i]));
-        if (k >= 1) {
-          const T bpv = i > 0 ? b[i - 1] : bp;
-          e[i] = l_sub(l_sub(e[i], l_mul(r, l_sub(b[i], bpv))), l_mul(dt, j[i]));
-        }
-      }
-    }
-    s_e[t] = e[0];
-    __syncthreads();
-    en = t + 1 < (int)blockDim.x ? s_e[t + 1] : T(0);
-#pragma unroll
-    for (int i = 0; i < C; ++i) {
-      const T enx = i + 1 < C ? e[i + 1] : en;
-      if (base + i < nz - 1) b[i] = l_sub(b[i], l_mul(hr, l_sub(enx, e[i])));
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < C; ++i) {
-    const int k = base + i;
-    if (k < nz) {
-      Eg[k] = e[i];
-      Bg[k] = b[i];
-      Jg[k] = j[i];
-    }
+// ------------------------------------------------------------- split line
+// Constants of the split float line, made on the host: the pulse along the
+// line in turns and in the envelope's own scale.
+struct SplitArgs {
+  LineArgs line;
+  StepBase base;            // carrier phase and time of step n (make_step_base)
+  FastPulse fast;           // s_env (here of the scaled argument below), turn0
+  int env, g;               // envelope kind; order of the super-Gaussian (Gaussian: 1)
+  float zs_hi, zs_lo;       // k / 2 pi
+  float zf_hi, zf_lo;
+  float su_vg;              // scale of the envelope argument over v_g
+  float hu;                 // dt/2 in the scaled argument
+  float env_w;              // half-width of the sin^2 window, scaled
+  float amp, jamp;          // a0, and the amplitude of J1
+  float delta;              // omega dt/2
+  float k1, k2;             // th = k1 u q, A = 1 - th^2/2 + k2 q
+};
+
+// Envelope form of a split-line kernel: the order g of the super-Gaussian where
+// it is compiled in (1: Gaussian and continuous wave), any order, or the sin^2
+// window.  The envelope is 2^-(u^{2g}) of the scaled argument u.
+constexpr int kOrderAny = 0, kSin2 = -1;
+
+// s^n, n >= 1; N > 0: n = N, by squaring
+template <int N>
+__device__ __forceinline__ F2 upow(F2 s, int n) {
+  if constexpr (N == 0) {
+    F2 p = s;
+    for (int i = 1; i < n; ++i) p = rmul(p, s);
+    return p;
+  } else if constexpr (N == 1) {
+    return s;
+  } else if constexpr (N % 2 == 0) {
+    return upow<N / 2>(rmul(s, s), 0);
+  } else {
+    return rmul(upow<N - 1>(s, 0), s);
   }
 }
+__device__ __forceinline__ F2 window2(F2 u, float w) {
+  const F2 c = cos_r(u);
+  return sin2_window(rmul(c, c), u, w);
+}
 
-template <typename T, int C, int MAXT>
-int launch_plasma_reg(const LineArgs &a, void *stream) {
-  const int block = ((a.nz + C - 1) / C + 31) / 32 * 32;
-  if (block > MAXT) return AP_ERR_ARG;
-  plasma_line_reg_kernel<T, C, MAXT><<<(unsigned)a.n_lines, block, 0, static_cast<cudaStream_t>(stream)>>>(a);
+// The split line of Sec. 4 in registers: E2, B2 and J of two runs of C nodes
+// per thread (ap_lines.cuh), each node's phase and envelope constants and a_k in
+// shared memory.  Per step and node the analytic E1 at t_n and J1 at t_n + dt/2:
+//   E1 = a0 G(eta) cos(psi),
+//   J1 = J0 G(eta') A sin(psi + omega dt/2 + th),  th = L1/omega,
+// where psi + omega dt/2 is J1's carrier and th the finite-duration phase
+// (Eq. j1), so one sine takes the place of a rotation, a sine, a cosine and a
+// complex product: four special-function operations per node instead of six.
+// The carrier phase is kept in turns, a node's share reduced once per launch.
+// The two B half steps that meet between E updates are one whole step.  34
+// packed operations per pair of nodes against about 75 (149 instructions per
+// node-step with the line in shared memory).
+// 304 lines of 4096 nodes, 500 steps: 3.10 -> 0.83 ms.
+template <int C, int MAXT, int G>
+__global__ void __launch_bounds__(MAXT) split_line_kernel(const __grid_constant__ SplitArgs sa) {
+  __shared__ float s_b[2 * MAXT + 1], s_e[2 * MAXT + 1];
+  extern __shared__ __align__(16) unsigned char s_split[];
+  F2 *s_turn = reinterpret_cast<F2 *>(s_split);  // [C][block] each
+  const LineArgs &a = sa.line;
+  const int nz = a.nz, t = threadIdx.x, bd = blockDim.x, H = C * bd;
+  F2 *s_eta = s_turn + C * bd, *s_q = s_eta + C * bd;
+  const size_t off = (size_t)blockIdx.x * (size_t)nz;
+  float *Eg = static_cast<float *>(a.E) + off;
+  float *Bg = static_cast<float *>(a.B) + off;
+  float *Jg = static_cast<float *>(a.J) + off;
+  const float *W = a.wp2 ? static_cast<const float *>(a.wp2) + off : nullptr;
+  const float dtf = (float)a.dt, rf = (float)(a.dt / a.dz);
+  const LineEdge eb{s_b}, ee{s_e};
+  F2 e[C], b[C], j[C];
+  line_load<C>(e, Eg, nz);
+  line_load<C>(b, Bg, nz);
+  line_load<C>(j, Jg, nz);
+  LineEnds ends;
+  ends.init<C>(nz, b);
+  const float e0 = e[0].x;
+#pragma unroll 1
+  for (int i = 0; i < C; ++i) {
+    F2 q, tn, en2;
+    for (int h = 0; h < 2; ++h) {
+      const int k = t * C + i + (h ? H : 0);
+      // z_k - z_f and its turns, float-float
+      const FF zk = node_coord_ff((float)k, a.z0_hi, a.z0_lo, a.dz_hi, a.dz_lo);
+      FF dz = two_sum(zk.hi, -sa.zf_hi);
+      dz.lo = __fadd_rn(dz.lo, __fsub_rn(zk.lo, sa.zf_lo));
+      FF tr = two_prod(sa.zs_hi, dz.hi);
+      tr.lo = __fadd_rn(tr.lo, __fmaf_rn(sa.zs_hi, dz.lo, __fmul_rn(sa.zs_lo, dz.hi)));
+      const float turn = __fadd_rn(__fsub_rn(tr.hi, round_magic(tr.hi)), tr.lo);
+      const float ek = __fmul_rn(sa.su_vg, __fadd_rn(dz.hi, dz.lo));
+      const float qk = __fmul_rn(dtf, k < nz ? (W ? W[k] : (float)a.omega_p2) : 0.0f);
+      if (h) { tn.y = turn; en2.y = ek; q.y = qk; } else { tn.x = turn; en2.x = ek; q.x = qk; }
+    }
+    s_turn[i * bd + t] = tn;
+    s_eta[i * bd + t] = en2;
+    s_q[i * bd + t] = q;
+  }
+  const F2 nr = F2(-rf), ndt = F2(-dtf);
+  auto b_step = [&](F2 en, F2 nh) {
+#pragma unroll
+    for (int i = 0; i < C; ++i) b[i] = rfma(nh, rsub(i + 1 < C ? e[i + 1 < C ? i + 1 : i] : en, e[i]), b[i]);
+    ends.restore<C>(b);
+  };
+  ee.put(e[0]);
+  __syncthreads();
+  b_step(ee.next(), F2(-0.5f * rf));
+  float nf = 0.0f;  // the step in float (exact: fewer than 2^23 steps)
+  for (long long n = 0; n < a.n_steps; ++n, nf += 1.0f) {
+    eb.put(b[C - 1]);
+    __syncthreads();
+    const F2 bp = eb.prev();
+    const float4 st = step_entry<AP_PLANE>(sa.fast, sa.base, nf);
+    F2 bq = bp;  // B before node i
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+      // psi = C - the node's turns, reduced
+      F2 turn = rsub(F2(st.x), s_turn[i * bd + t]);
+      turn = rsub(turn, round_magic(turn));
+      const F2 u0 = rsub(F2(st.y), s_eta[i * bd + t]), u1 = radd(u0, F2(sa.hu));
+      F2 m0, m1, th = F2(0.0f), A = F2(1.0f);
+      if constexpr (G == kSin2) {
+        m0 = window2(u0, sa.env_w);
+        m1 = window2(u1, sa.env_w);
+      } else {
+        m0 = exp2_neg(upow<G>(rmul(u0, u0), sa.g));
+        const F2 s = rmul(u1, u1);
+        if constexpr (G == 1) {
+          m1 = exp2_neg(s);
+          th = rmul(F2(sa.k1), u1);
+          A = rfma(rmul(F2(-0.5f), th), th, F2(1.0f + sa.k2));
+        } else {
+          F2 q = F2(1.0f);
+          if (G > 1 || sa.g > 1) q = upow<(G > 1 ? G - 1 : 0)>(s, sa.g - 1);
+          m1 = exp2_neg(rmul(q, s));
+          th = rmul(F2(sa.k1), rmul(u1, q));
+          A = rfma(F2(sa.k2), q, rfma(rmul(F2(-0.5f), th), th, F2(1.0f)));
+        }
+      }
+      const F2 c0 = cos_r(rmul(turn, F2(kTwoPiHi)));
+      const F2 aj = rfma(turn, F2(kTwoPiHi), radd(th, F2(sa.delta)));
+      const F2 sj = F2(mufu_sin(aj.x), mufu_sin(aj.y));
+      // J^{n+1/2} = J^{n-1/2} + a_k (E1 + E2)^n;  E^{n+1} = (E^n - r dB) - dt (J - J1)^{n+1/2}
+      j[i] = rfma(s_q[i * bd + t], rfma(F2(sa.amp), rmul(m0, c0), e[i]), j[i]);
+      const F2 src = rfma(rmul(F2(-sa.jamp), m1), rmul(A, sj), j[i]);
+      e[i] = rfma(ndt, src, rfma(nr, rsub(b[i], bq), e[i]));
+      bq = b[i];
+    }
+    if (t == 0) e[0].x = e0;
+    ee.put(e[0]);
+    __syncthreads();
+    b_step(ee.next(), n + 1 < a.n_steps ? nr : F2(-0.5f * rf));
+  }
+  line_store<C>(e, Eg, nz);
+  line_store<C>(b, Bg, nz);
+  line_store<C>(j, Jg, nz);
+}
+
+template <int C, int MAXT, int G>
+int launch_split_g(const SplitArgs &sa, void *stream) {
+  auto kern = split_line_kernel<C, MAXT, G>;
+  const int block = line_block<C>(sa.line.nz);
+  const size_t smem = 3 * sizeof(F2) * (size_t)C * block;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return AP_ERR_CUDA;
+  kern<<<(unsigned)sa.line.n_lines, block, smem, static_cast<cudaStream_t>(stream)>>>(sa);
   return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
 }
 
-template <typename T, int PREC, bool APT>
-int launch_line_t(const Pulse<Real<PREC>> &P, const LineArgs &a, void *stream) {
-  auto kern = line_kernel<T, PREC, APT>;
-  const size_t per_node = 4u * sizeof(T) + ((APT && PREC == AP_FP32_PHASEFF) ? 3u * sizeof(float) : 0u);
-  const size_t smem = per_node * (size_t)a.nz;
+template <int C, int MAXT>
+int launch_split(const SplitArgs &sa, void *stream) {
+  if (sa.env == AP_ENV_SIN2) return launch_split_g<C, MAXT, kSin2>(sa, stream);
+  if (sa.g == 1) return launch_split_g<C, MAXT, 1>(sa, stream);
+  if (sa.g == 4) return launch_split_g<C, MAXT, 4>(sa, stream);
+  return launch_split_g<C, MAXT, kOrderAny>(sa, stream);
+}
+
+SplitArgs split_args(const Pulse<double> &pd, const Pulse<float> &pf, const LineArgs &a) {
+  SplitArgs s;
+  s.line = a;
+  s.fast = pf.fast;
+  s.env = pd.env;
+  // 2^-(u^{2g}) with u = su eta; the logarithmic derivatives are given in
+  // eta (Gaussian) or eta/tau (super-Gaussian), ratio: that argument over u
+  const double log2e = 1.4426950408889634;
+  double su = 0.0, ratio = 0.0;
+  s.g = 1;
+  if (pd.env == AP_ENV_GAUSS) {
+    su = std::sqrt(pd.env_a);
+    ratio = 1.0 / su;
+  } else if (pd.env == AP_ENV_SGAUSS) {
+    s.g = pd.sg_order;
+    const double sc = std::pow(log2e, 0.5 / s.g);  // env_a = 1/tau, env_b = log2e
+    su = pd.env_a * sc;
+    ratio = 1.0 / sc;
+  } else if (pd.env == AP_ENV_SIN2) {
+    su = pd.env_a;
+  }
+  s.fast.s_env = (float)su;
+  s.fast.c_tz = 0.0f;
+  GridView none;
+  std::memset(&none, 0, sizeof(none));
+  s.base = make_step_base(pf, a.t0, a.dt, none);
+  auto split = [](double v, float &hi, float &lo) {
+    hi = (float)v;
+    lo = (float)(v - (double)hi);
+  };
+  split(pf.fast.z_scale, s.zs_hi, s.zs_lo);
+  s.zf_hi = pf.zf_hi;
+  s.zf_lo = pf.zf_lo;
+  s.su_vg = (float)(su * pd.inv_vg);
+  s.hu = (float)(0.5 * a.dt * su);
+  s.env_w = (float)(pd.env_a * pd.env_b);
+  s.amp = (float)pd.amp;
+  s.jamp = (float)(pd.jamp * pd.amp);
+  s.delta = (float)(0.5 * pd.omega * a.dt);
+  s.k1 = (float)(-pd.lg_c1 * pd.inv_w * std::pow(ratio, 2.0 * s.g - 1.0));
+  s.k2 = (float)(pd.lg_c2 * pd.inv_w * pd.inv_w * std::pow(ratio, 2.0 * s.g - 2.0));
+  if (pd.env != AP_ENV_GAUSS && pd.env != AP_ENV_SGAUSS) s.k1 = s.k2 = 0.0f;
+  return s;
+}
+
+template <typename T, bool APT>
+int launch_line_t(const Pulse<double> &P, const LineArgs &a, void *stream) {
+  auto kern = line_kernel<T, APT>;
+  const size_t smem = 4u * sizeof(T) * (size_t)a.nz;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return AP_ERR_CUDA;
   int block = (a.nz + 31) / 32 * 32;
@@ -320,18 +360,23 @@ int launch_line_t(const Pulse<Real<PREC>> &P, const LineArgs &a, void *stream) {
 
 int launch_line(bool apt_mode, int precision, const Pulse<double> &pd, const Pulse<float> &pf,
                 const LineArgs &a, void *stream) {
-  // traditional float lines up to 8 x 768 nodes: the line in registers
-  if (!apt_mode && precision != AP_FP64) {
-    if (a.nz <= kLineBlock) return launch_plasma_reg<float, 1, kLineBlock>(a, stream);
-    if (a.nz <= 2 * kLineBlock) return launch_plasma_reg<float, 2, kLineBlock>(a, stream);
-    if (a.nz <= 4 * kLineBlock) return launch_plasma_reg<float, 4, kLineBlock>(a, stream);
-    if (a.nz <= 8 * 768) return launch_plasma_reg<float, 8, 768>(a, stream);
+  if (precision != AP_FP64) {
+    // the line in registers, two runs of C nodes per thread
+    if (apt_mode) {
+      const SplitArgs s = split_args(pd, pf, a);
+      // measured at 1 to 304 lines: shorter runs (more threads) while the
+      // barriers weigh most, longer ones as the line grows (304 lines, 60
+      // steps, C = 1/2/4/8: 700 nodes 68/65/73/75 us, 2000 nodes
+      // 116/107/95/97, 4096 nodes -/-/148/150)
+      if (a.nz <= 512) return launch_split<1, 256>(s, stream);
+      if (a.nz <= 1536) return launch_split<2, 384>(s, stream);
+      if (a.nz <= 4096) return launch_split<4, 512>(s, stream);
+      return launch_split<8, 512>(s, stream);
+    }
+    if (a.nz <= kPlasmaPairNodes) return launch_plasma_float(a, stream);
+    return launch_line_t<float, false>(pd, a, stream);
   }
-  if (precision == AP_FP64)
-    return apt_mode ? launch_line_t<double, AP_FP64, true>(pd, a, stream)
-                    : launch_line_t<double, AP_FP64, false>(pd, a, stream);
-  return apt_mode ? launch_line_t<float, AP_FP32_PHASEFF, true>(pf, a, stream)
-                  : launch_line_t<float, AP_FP32_PHASEFF, false>(pf, a, stream);
+  return apt_mode ? launch_line_t<double, true>(pd, a, stream) : launch_line_t<double, false>(pd, a, stream);
 }
 
 }  // namespace apt
