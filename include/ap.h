@@ -254,7 +254,9 @@ typedef struct {
 #define AP_APT1D_MAX_NODES_F32 8192   /* nodes per float line of ap_apt1d_run (it also keeps
                                          three per-node phase constants in shared memory) */
 
-/* Launch shape, chosen by the autotuner (0 = library default). */
+/* Launch shape, chosen by the autotuner (block 0 = library default).  While
+ * none is set, the library picks block, pairs and grid_cache by the call's
+ * size, arithmetic and grid layout. */
 typedef struct {
   int32_t block;          /* threads per block, multiple of 32, <= 1024 */
   int32_t blocks_per_sm;  /* persistent kernels: resident blocks per SM */
@@ -268,7 +270,7 @@ typedef struct {
                              grid: 1 = each thread carries two particles, every FP32 operation
                              of the field, the Boris step and the position packed (f32x2) over
                              the pair; 0 = one particle per thread.  Results do not depend on
-                             the launch shape within either setting. */
+                             the launch shape. */
   int32_t tile;           /* batched launch: particles per tile, a multiple of the particles
                              a block carries (block x (1 + pairs)); 0 = one block's worth */
 } ap_launch_cfg;

@@ -18,10 +18,9 @@ over the caller's own set mix.  The dimensions searched:
 
 Results are cached in a JSON file keyed by GPU name, the library build (a
 hash of libapt.so, so that a rebuilt kernel is tuned afresh), kind,
-precision, grid layout and a size bucket.  Within one particles-per-thread
-setting every shape gives bit-identical particle states (the per-particle
-arithmetic does not depend on the launch); the one- and two-particle kernels
-differ only in float rounding.
+precision, grid layout and a size bucket.  Every shape gives bit-identical
+particle states: the per-particle arithmetic depends neither on the launch nor
+on the particles per thread.
 """
 import hashlib
 import json

@@ -25,6 +25,7 @@ struct ap_handle_s {
   Pulse<float> *d_pf = nullptr;
   int *d_status = nullptr;
   apt::LaunchShape shape{0, 0, 0, 0, 0};
+  bool shape_set = false;  // by ap_set_launch: otherwise default_shape picks
 };
 
 struct ap_graph_s {
@@ -502,12 +503,43 @@ int make_diag(const ap_diag *d, long long n_steps, int n_sets, apt::DiagView &v,
   return AP_OK;
 }
 
-int default_block(const ap_handle_s *h, long long n) {
+int default_block(const ap_handle_s *h, long long n, int precision) {
   if (h->shape.block > 0) return h->shape.block;
+  // FP64: a warp's double instruction holds its scheduler's unit for 64 cycles
+  // whatever the number of its lanes, so whole warps are spread as evenly as
+  // they go (100 steps of 2e4 plane-wave electrons: 861 us with blocks of 128,
+  // 687 with 64, 623 with 32; 3e4: 908, 887, 790)
+  if (precision == AP_FP64) return 32;
   long long per_sm = n / (h->sm_count > 0 ? h->sm_count : 1);
   int b = 128;
   while (b > 32 && per_sm < b) b >>= 1;
   return b;
+}
+
+// The launch shape of a float-float push that ap_set_launch left open (every
+// shape gives the same bits).  Measured on the Gaussian beam, the LG beam and
+// the flying focus, 1e3 to 4e6 particles:
+//   - per-cell coefficients: one particle per thread with its cell in
+//     registers, in blocks of 256 from about 1500 particles per SM (256^3 grid,
+//     200 steps, cell in shared memory / this / two particles per thread: 1e5
+//     288 / 243 / 263 us, 1e6 1506 / 1309 / 1388, 4e6 5545 / 4796 / 4934);
+//   - no grid: two particles per thread from 640 per SM, where both halves
+//     still leave every scheduler warps (100 steps, one / two: LG 1e5
+//     157 / 146 us, Gaussian 1e5 118 / 115, 1e6 376 / 361, 3e6 992 / 915; below,
+//     one is as fast or faster: LG 1e4 115 / 119);
+//   - batched, no grid: two from 2048 per SM (256 sets, 6e5 311 / 285 us; 64
+//     sets, 2e5 174 / 183).
+void default_shape(const ap_handle_s *h, long long n, int precision, bool batched, apt::PushArgs &a) {
+  if (h->shape_set || precision != AP_FP32_PHASEFF) return;
+  const long long per_sm = n / (h->sm_count > 0 ? h->sm_count : 1);
+  if (a.grid_on) {
+    if (!a.grid.cells) return;
+    a.shape.grid_cache = 1;
+    if (per_sm >= 1536) a.shape.block = 256;
+  } else if (per_sm >= (batched ? 2048 : 640)) {
+    a.shape.pairs = 1;
+    a.shape.block = 64;
+  }
 }
 
 int fill_push_args(ap_handle_s *h, const ap_particles *p, const ap_grid *g, double t0, double dt,
@@ -541,7 +573,8 @@ int fill_push_args(ap_handle_s *h, const ap_particles *p, const ap_grid *g, doub
   a.status = h->d_status;
   a.sm_count = h->sm_count;
   a.shape = h->shape;
-  a.shape.block = default_block(h, p->n);
+  a.shape.block = default_block(h, p->n, precision);
+  default_shape(h, p->n, precision, false, a);
   return AP_OK;
 }
 
@@ -701,6 +734,7 @@ int ap_set_launch(ap_handle h, const ap_launch_cfg *cfg) {
   if (!h) return AP_ERR_ARG;
   if (!cfg) {
     h->shape = apt::LaunchShape{0, 0, 0, 0, 0};
+    h->shape_set = false;
     return AP_OK;
   }
   if (cfg->block != 0 && (cfg->block < 32 || cfg->block > 256 || (cfg->block & 31))) return AP_ERR_ARG;
@@ -709,6 +743,7 @@ int ap_set_launch(ap_handle h, const ap_launch_cfg *cfg) {
   if (cfg->pairs != 0 && cfg->pairs != 1) return AP_ERR_ARG;
   if (cfg->tile < 0 || cfg->tile > (1 << 24)) return AP_ERR_ARG;
   h->shape = apt::LaunchShape{cfg->block, cfg->blocks_per_sm, cfg->grid_cache, cfg->pairs, cfg->tile};
+  h->shape_set = true;
   return AP_OK;
 }
 
@@ -823,9 +858,11 @@ int ap_gather_push_batched(ap_handle h, const ap_particles *p, const ap_grid *g,
   rc = fill_push_args(h, p, g, t0, dt, n_steps, precision, diag, h->n_sets, ba.base, stream);
   if (rc != AP_OK) return rc;
   if (n_steps == 0) return AP_OK;
+  ba.base.shape = h->shape;
   ba.base.shape.block = h->shape.block > 0 ? h->shape.block : 128;
+  default_shape(h, p->n, precision, true, ba.base);
   // particles per tile: a multiple of what one block carries per pass
-  const int per_pass = ba.base.shape.block * (h->shape.pairs ? 2 : 1);
+  const int per_pass = ba.base.shape.block * (ba.base.shape.pairs ? 2 : 1);
   if (h->shape.tile > 0 && h->shape.tile % per_pass != 0) return AP_ERR_ARG;
   ba.set_offsets = reinterpret_cast<const long long *>(p->set_offsets);
   ba.n_sets = h->n_sets;
