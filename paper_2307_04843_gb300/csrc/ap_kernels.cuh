@@ -142,6 +142,143 @@ __device__ __forceinline__ double push_one(const Pulse<Real<PREC>> &P, const Pus
                               1.0));
 }
 
+// The FP64 push without a grid of plane waves and Gaussian beams.  A double
+// instruction holds a scheduler's unit for 64 cycles, so a step costs its
+// instructions: the polarisation is a compile-time parameter (in the pulse's
+// frame, as in push_ff), so that zero components and the unused half of a sine
+// and cosine are not evaluated, and the Boris step is boris_unit (kick and
+// rotation summed before they join the momentum).  Arguments and result as for
+// push_one.  1e4 electrons in a plane wave, 2000 steps with the light-front
+// diagnostic: 9.96 -> 6.62 ms.
+template <int KIND>
+constexpr bool kPushD = KIND == AP_PLANE || KIND == AP_GAUSS || KIND == AP_FLYING_CF;
+
+struct KickD {
+  double hA, hAbr, hAce, hAcb, kA, kAce;
+};
+
+template <int KIND, int POL>
+__device__ __forceinline__ UnitFields<double> unit_fields_d(const Pulse<double> &P, const Local<double> &L) {
+  UnitFields<double> f;
+  double mul, l2;
+  envelope(P, L.eta, mul, l2);
+  if constexpr (KIND == AP_PLANE) {
+    double mag = mul;
+    if (l2 != 0.0) mag *= exp2(l2);
+    if (POL == kLin && !P.plasma) {
+      f.Ur = mag * cos(L.psi);
+      f.Ui = 0.0;
+    } else {
+      double s, c;
+      sincos(L.psi, &s, &c);
+      f.Ur = mag * c;
+      f.Ui = mag * s;
+    }
+    f.Vr = f.Ur;
+    f.Vi = f.Ui;
+    if (P.plasma) {
+      double L1, L2;
+      envelope_logd(P, L.eta, L1, L2);
+      const Cx<double> V = finite_duration(Cx<double>{f.Ur, f.Ui}, P.fdc, L1, L2, P.inv_w);
+      f.Vr = V.re;
+      f.Vi = V.im;
+    }
+    f.ez = f.bz = 0.0;
+  } else {
+    const BeamZ<double> Z = gauss_z<KIND == AP_FLYING_CF>(P, L);
+    const double a = (L.x * L.x + L.y * L.y) * P.inv_w0sq;
+    const double mag = mul * exp2(fma(a * Z.q.re, -kLog2e, l2));
+    double s, c;
+    sincos(L.psi - a * Z.q.im, &s, &c);
+    const Cx<double> U = cmul(Z.q, Cx<double>{mag * c, mag * s});
+    f.Ur = f.Vr = U.re;
+    f.Ui = f.Vi = U.im;
+    f.ez = f.bz = 0.0;
+    if (P.lon) {
+      const Cx<double> W = cmul(Z.q, U);
+      f.ez = POL == kLin ? L.x * W.im : fma(L.x, W.im, -(L.y * W.re));
+      f.bz = POL == kLin ? L.y * W.im : fma(L.x, W.re, L.y * W.im);
+    }
+  }
+  return f;
+}
+
+template <int KIND>
+__device__ __forceinline__ double push_d(const Pulse<double> &P, const PushArgs &a, long long i, bool valid) {
+  double *uxs = static_cast<double *>(a.ux), *uys = static_cast<double *>(a.uy), *uzs = static_cast<double *>(a.uz);
+  const int frame = P.fast.frame;
+  Pos<AP_FP64> pos;
+  double u[3] = {0.0, 0.0, 0.0};
+  pos.load(0.0, 0.0, 0.0);
+  if (valid) {
+    pos.load(a.x[i], a.y[i], a.z[i]);
+    u[0] = uxs[i];
+    u[1] = uys[i];
+    u[2] = uzs[i];
+    if (frame == 1) {
+      const double t = pos.x, tu = u[0];
+      pos.x = pos.y;
+      pos.y = -t;
+      u[0] = u[1];
+      u[1] = -tu;
+    } else if (frame == 2) {
+      pos.y = -pos.y;
+      u[1] = -u[1];
+    }
+  }
+  const double dt = a.dt, dtxy = dt * P.adv_xy, h = -0.5 * dt, g = P.lon ? -2.0 * P.inv_w0sq : 0.0;
+  KickD k;
+  k.hA = h * P.amp;
+  k.hAbr = k.hA * P.bratio;
+  k.hAce = k.hA * P.lonE * g;
+  k.hAcb = k.hAbr * P.lonB * g;
+  k.kA = 2.0 * k.hA;
+  k.kAce = 2.0 * k.hAce;
+  // gamma from 1 + u^2 and its inverse root (no division)
+  auto gamma_of = [&](double ig) { return fma(u[0], u[0], fma(u[1], u[1], fma(u[2], u[2], 1.0))) * ig; };
+  const double h0 = gamma_of(inv_gamma(u)) - u[2];
+  double *lf = a.diag.lf;
+  auto steps = [&](auto pol_c, auto lf_c) {
+    constexpr int POL = decltype(pol_c)::value;
+    constexpr bool LF = decltype(lf_c)::value;
+    double nd = 0.0;
+    for (long long n = 0; n < a.n_steps; ++n, nd += 1.0) {
+      const Local<double> L = local_coords<AP_FP64>(P, fma(nd, dt, a.t0), pos);
+      const UnitFields<double> f = unit_fields_d<KIND, POL>(P, L);
+      const double ig = boris_unit<POL, KIND != AP_PLANE>(u, f, k);
+      pos.advance(u[0] * ig, u[1] * ig, u[2] * ig, dtxy, dt);
+      if constexpr (LF) warp_max_to(lf + n, valid ? fabs((gamma_of(ig) - u[2]) - h0) : 0.0, 0xffffffffu);
+    }
+  };
+  using Lin = std::integral_constant<int, kLin>;
+  using Circ = std::integral_constant<int, kCirc>;
+  if (P.fast.circ) {
+    if (lf) steps(Circ{}, std::true_type{});
+    else steps(Circ{}, std::false_type{});
+  } else {
+    if (lf) steps(Lin{}, std::true_type{});
+    else steps(Lin{}, std::false_type{});
+  }
+  if (!valid) return 0.0;
+  if (frame == 1) {
+    const double t = pos.x, tu = u[0];
+    pos.x = -pos.y;
+    pos.y = t;
+    u[0] = -u[1];
+    u[1] = tu;
+  } else if (frame == 2) {
+    pos.y = -pos.y;
+    u[1] = -u[1];
+  }
+  pos.store(a.x + i, a.y + i, a.z + i);
+  uxs[i] = u[0];
+  uys[i] = u[1];
+  uzs[i] = u[2];
+  if (!all_finite(pos.x, pos.y, pos.z, u[0], u[1], u[2])) atomicOr(a.status, kStatusNonfinite);
+  return __dsqrt_rn(__dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(u[0], u[0]), __dmul_rn(u[1], u[1])), __dmul_rn(u[2], u[2])),
+                              1.0));
+}
+
 // One or two particles of a thread (R = float or F2) through n_steps fused
 // float-float steps (ap_step.cuh): load (a2), per step the phase and unit
 // fields (a3-a7), grid gather (a8), Boris and position (a9), light-front
@@ -479,7 +616,8 @@ template <int KIND, int PREC, int GRID>
 __device__ __forceinline__ void push_body(const Pulse<Real<PREC>> &P, const PushArgs &a, unsigned hist_off) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   push_chunks<1>(a, s_dyn, hist_off, [&](long long i, double g[2]) {
-    g[0] = push_one<KIND, PREC, GRID>(P, a, i, i < a.n, s_dyn + step_table_bytes(blockDim.x));
+    if constexpr (PREC == AP_FP64 && GRID == kGridNone && kPushD<KIND>) g[0] = push_d<KIND>(P, a, i, i < a.n);
+    else g[0] = push_one<KIND, PREC, GRID>(P, a, i, i < a.n, s_dyn + step_table_bytes(blockDim.x));
   });
 }
 
@@ -653,7 +791,9 @@ __device__ __forceinline__ void batch_body(const Pulse<Real<PREC>> *__restrict__
         if (valid) acc += g[0];
         if (valid1) acc += g[1];
       } else {
-        double g = push_one<KIND, PREC, GRID>(sp, a, i, valid, slots);
+        double g;
+        if constexpr (PREC == AP_FP64 && GRID == kGridNone && kPushD<KIND>) g = push_d<KIND>(sp, a, i, valid);
+        else g = push_one<KIND, PREC, GRID>(sp, a, i, valid, slots);
         if (valid) acc += g;
       }
     }

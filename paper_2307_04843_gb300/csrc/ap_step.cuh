@@ -55,6 +55,13 @@ __device__ __forceinline__ float sin2_window(float m, float eta, float b) { retu
 __device__ __forceinline__ FF two_diff(float a, float b) { return two_sum(a, -b); }
 __device__ __forceinline__ float clamp_abs(float a, float b) { return fminf(fmaxf(a, -b), b); }
 
+// double: the FP64 push's Boris step (push_d); sums of products contract by
+// themselves
+__device__ __forceinline__ double rmul(double a, double b) { return a * b; }
+__device__ __forceinline__ double radd(double a, double b) { return a + b; }
+__device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double rneg(double a) { return -a; }
+
 namespace pair {
 __device__ __forceinline__ F2 rmul(F2 a, F2 b) { return a * b; }
 __device__ __forceinline__ F2 radd(F2 a, F2 b) { return a + b; }
@@ -510,8 +517,8 @@ __device__ __forceinline__ R inv_gamma(const R u[3]) {
 
 // the analytic field alone, from its unit fields and the kick's constants
 // (LON: the kind has longitudinal fields); returns 1/gamma of the new momentum
-template <int POL, bool LON, typename R>
-__device__ __forceinline__ R boris_unit(R u[3], const UnitFields<R> &f, const StepBase &s) {
+template <int POL, bool LON, typename R, class S>
+__device__ __forceinline__ R boris_unit(R u[3], const UnitFields<R> &f, const S &s) {
   R um[3] = {rfma(R(s.hA), f.Ur, u[0]), u[1], u[2]};
   if constexpr (POL == kCirc) um[1] = rfma(R(s.hA), f.Ui, u[1]);
   if constexpr (LON) um[2] = rfma(R(s.hAce), f.ez, u[2]);
