@@ -708,9 +708,9 @@ struct PairIO {
 struct RevConst {
   float hbr, hce, hcb;    // h times B0/E0, the E_z and the B_z factor
   float dxy, dt;          // position increments per unit velocity
-  float w2, zr, k, eta;   // 2/w0^2, 1/z_R, k, and 2 ln2 s_env / v_g, times a0
-  float a0, vg;           // a0; a0 / v_g (envelopes other than the Gaussian)
-  float zr1, omb;         // 1/z_R and 1/(1 - beta_f)
+  float w2, a0;           // 2 a0/w0^2, a0
+  float zr, k, eta, vg;   // 1/z_R, k, 2 ln2 s_env / v_g (Gaussian envelope), 1/v_g
+  float omb;              // 1/(1 - beta_f)
 };
 
 // Gamma'/Gamma of the envelope at eta s_env (see envelope_dlog), times 1: the
@@ -753,7 +753,7 @@ __device__ __forceinline__ F2 dlog_scaled(const PT &P, F2 e, F2 mul) {
 //   (Gamma'/Gamma) Re Y, -Im Y,
 // formed once, and each direction (x, y, z - z_f, w0, beta_f) is a short real
 // combination of them.  Re Y is also F . f, the derivative in a0.
-// gr: d/da0, -(w0/2) d/dw0 / a0, d/dz_f, d/dbeta_f / a0.
+// gr: d/da0, (w0/2) d/dw0 / a0, d/dz_f / a0, d/dbeta_f / a0.
 template <int KIND, int POL, int ENV, class PT>
 __device__ __forceinline__ void reverse_step_pair(const PT &P, const StepBase &sb, const RevConst &rc, const float4 st,
                                                   F2 x, F2 y, F2 zhi, F2 zlo, const F2 u[3], F2 lx[3], F2 lu[3],
@@ -885,12 +885,14 @@ __device__ __forceinline__ void reverse_step_pair(const PT &P, const StepBase &s
   R dz = rfma(R(rc.k), Yi, rmul(R(rc.zr), Sz));
   if constexpr (ENV == kEnvGauss) dz = rfma(rmul(R(rc.eta), eta), Yr, dz);
   else dz = rfma(rmul(R(-rc.vg), dlog_scaled(P, eta, mul)), Yr, dz);
-  lx[2] = radd(lx[2], dz);
+  // per unit amplitude: k = 1 stays exact (a rounded k a0 would shift the whole
+  // carrier part of d/dz_f, which cancels to a small rest over the particles)
+  lx[2] = rfma(R(rc.a0), dz, lx[2]);
   gr[0] = radd(gr[0], Yr);
   gr[1] = rfma(Pr, a, rfma(Sz, zn, rsub(gr[1], Zr)));
   gr[2] = rsub(gr[2], dz);
   if constexpr (KIND == AP_FLYING_CF)
-    gr[3] = rfma(Sz, rfma(zn, R(-rc.omb), R(-rc.zr1 * st.w)), gr[3]);
+    gr[3] = rfma(Sz, rfma(zn, R(-rc.omb), R(-rc.zr * st.w)), gr[3]);
 }
 
 template <int KIND>
@@ -944,11 +946,17 @@ __global__ void __launch_bounds__(kAdjBlock, kAdjPairBlocksPerSm)
       if (threadIdx.x == 0) {
         s_set = set;
         s_base = make_step_base(P, a.t0, a.dt, a.grid);
+        const FastPulse &F = P.fast;
         const float g = P.lon ? -2.0f * P.inv_w0sq : 0.0f, a0 = P.a0, h = s_base.h;
+        // the derivatives' constants from the rounded ones of the step itself, so
+        // that the reverse differentiates the map that ran (the terms of d/dz_f
+        // cancel to a small rest)
+        const double eta_z = (double)F.c_eta * F.z_scale;  // d(eta s_env)/dz
         s_rev = RevConst{h * P.bratio, h * P.lonE * g, h * P.bratio * P.lonB * g,
-                         (float)a.dt * P.adv_xy, (float)a.dt,
-                         2.0f * P.inv_w0sq * a0, P.inv_zR * a0, (float)P.k * a0,
-                         1.38629436f * P.fast.s_env * P.inv_vg * a0, a0, P.inv_vg * a0, P.inv_zR, P.inv_1mb};
+                         (float)a.dt * P.adv_xy, (float)((double)s_base.cz * F.z_len),
+                         (float)(2.0 * 0.69314718055994531 * (double)F.c_a) * a0, a0,
+                         (float)(-(double)F.c_zn * F.z_scale), (float)P.k,
+                         (float)(-2.0 * 0.69314718055994531 * eta_z), (float)(-eta_z / (double)F.s_env), P.inv_1mb};
       }
     }
     __syncthreads();
@@ -1062,6 +1070,7 @@ __global__ void __launch_bounds__(kAdjBlock, kAdjPairBlocksPerSm)
     else if (P.env == AP_ENV_GAUSS) sweep(Lin{}, EnvG{});
     else sweep(Lin{}, EnvA{});
     gacc[1] *= 2.0 * (double)P.inv_w0 * (double)P.a0;
+    gacc[2] *= (double)P.a0;
     gacc[3] *= (double)P.a0;
 
     if ((v0 || v1) && !(isfinite(gacc[0]) && isfinite(gacc[1]) && isfinite(gacc[2]) && isfinite(gacc[3])))
