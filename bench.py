@@ -44,33 +44,33 @@ MUFU_LANES = 16       # special-function operations per clock per SM
 SM_MAX_MHZ = 2070.0
 
 # FP32-pipe operations per particle-step, counted from the formulas each
-# kernel evaluates, and MUFU operations.
-# Workload 2 (Gaussian + longitudinal + grid, float-float phase): local
-# coordinates and phase 34, envelope 2, Gaussian profile + longitudinal +
-# assembly 28, trilinear gather from the cached cell 57, Boris 42,
-# compensated position update 18, z for the gather 1.
+# kernel evaluates (the float-float step of csrc/ap_step.cuh), and MUFU
+# operations.  Gaussian beam, linear polarisation, longitudinal terms: unit
+# fields 29 (carrier phase 9 of them), Boris step 29, position update 14.
+# Workload 2 adds the grid: unit fields 29, grid units and cell test 9,
+# trilinear gather 42, assembly 4, Boris step for any field 38, position 14.
+# Workload 3 (CP LG_{1,2}): unit fields 70, Boris 39, position 14.  Workload 4:
+# 18.5 per component, 75 per step.
 ALGO = {
     1: dict(fp32=0, mufu=0, fp64=60),
-    2: dict(fp32=182, mufu=7),
-    3: dict(fp32=190, mufu=8),
-    4: dict(fp32=2300, mufu=258),
-    5: dict(fp32=125, mufu=7),
-    6: dict(fp32=125, mufu=7),
+    2: dict(fp32=136, mufu=7),
+    3: dict(fp32=123, mufu=8),
+    4: dict(fp32=1259, mufu=227),
+    5: dict(fp32=72, mufu=7),
+    6: dict(fp32=72, mufu=7),
 }
 # FP32 operations per particle-step of the adjoint of workload 5 (Gaussian,
 # longitudinal terms, linear polarisation, no grid), from its formulas: the
-# forward sweep 125, the recomputation 125 and the reverse step 307 (local
-# coordinates and phase 34, envelope 2, field value 28, F = a0 f 4, the Boris
-# cotangent 123, the closed-form field derivatives contracted with it 116).
-ADJ_OPS = 557
+# forward sweep 72, the recomputation 72 and the reverse step 156 (unit fields
+# 31, the Boris reverse 81, cotangents and derivatives 44).
+ADJ_OPS = 300
 # DRAM bytes per particle-step of the workload-2 push kernel from the committed
 # ncu capture of the 1.6e6-particle x 4000-step case, scaled by particle-steps
 # (an upper bound at 1e7 particles: more particles share each cached cell);
-# None when the kernel changed after the capture.  The capture is of the
-# two-particle kernel with the hybrid cell cache (the autotuner's choice).
+# None when the kernel changed after the capture, as now.
 TRAFFIC_PER_PARTICLE_STEP = {
     "nodes": None,
-    "cells": 6.0486,  # (38.6484e9 read + 0.0626e9 written) / 6.4e9
+    "cells": None,
     "arrays": None,
 }
 TRAFFIC_KERNEL = dict(pairs=1, grid_cache=2)  # the launch setting the capture was taken with

@@ -1167,20 +1167,19 @@ __global__ void __launch_bounds__(256) nodes_row_kernel(const __grid_constant__ 
   }
 }
 
-// The row kernel with two nodes per lane and iteration (float-float, beams):
+// The row kernel with two nodes per lane and iteration (float-float, LG beams
+// and the flying-focus sum):
 // lane l takes x = l + 64 m and l + 64 m + 32, the two halves of every packed
 // value (ap_pair.cuh), so the position part of the six evaluations -- the
 // only per-node work -- issues once for both nodes.  Each warp takes a
 // contiguous run of rows, so the z/t part of its rows (carrier phase and
-// envelope argument; for Gaussian beams also the envelope and q) is computed
-// only when the z index changes, once per run of up to ny rows, instead of
-// once per row.  Stores stay coalesced: the warp writes 32 consecutive
+// envelope argument) is computed only when the z index changes, once per run
+// of up to ny rows, instead of once per row.  Stores stay coalesced: the warp writes 32 consecutive
 // elements for each half.
 template <int KIND, typename T>
 __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_constant__ Pulse<float> P,
                                                              const __grid_constant__ NodeArgs a) {
   using W = typename std::conditional<(sizeof(T) > sizeof(float)), T, float>::type;
-  constexpr bool kGaussZ = KIND == AP_GAUSS || KIND == AP_FLYING_CF;
   unsigned want = 0u;
   for (int q = 0; q < a.n_comp; ++q) want |= 1u << a.comp[q];
   const long long rows = (long long)a.ny * a.nz;
@@ -1196,7 +1195,6 @@ __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_consta
   constexpr int kOx[6] = {1, 0, 0, 0, 1, 1}, kOy[6] = {0, 1, 0, 1, 0, 1}, kOz[6] = {0, 0, 1, 1, 1, 0};
   int kcur = -1;
   Local<F2> Lz[2];
-  BeamZ<F2> Bz[2];
   // (j, k) of the run's first row by one division, then stepped row by row
   int k = (int)(r0 / a.ny);
   int j = (int)(r0 - (long long)k * a.ny);
@@ -1214,13 +1212,7 @@ __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_consta
         pos.y = FF{0.0f, 0.0f};
         pos.z = node_coord_ff((float)k + (h ? 0.5f : 0.0f), a.lo_hi[2], a.lo_lo[2], a.d_hi[2], a.d_lo[2]);
         const Local<float> l = local_coords<AP_FP32_PHASEFF>(P, st, pos);
-        if constexpr (kGaussZ) {
-          const BeamZ<float> b = gauss_z<KIND == AP_FLYING_CF>(P, l);
-          Bz[h] = BeamZ<F2>{Cx<F2>{F2(b.q.re), F2(b.q.im)}, F2(b.amp_mul), F2(b.l2), F2(b.psi)};
-        } else {
-          Lz[h] = Local<F2>{F2(l.x), F2(l.y), F2(l.dz), F2(l.psi), F2(l.eta), F2(l.T), F2(l.phi_hi),
-                            F2(l.phi_lo)};
-        }
+        Lz[h] = Local<F2>{F2(l.x), F2(l.y), F2(l.dz), F2(l.psi), F2(l.eta), F2(l.T), F2(l.phi_hi), F2(l.phi_lo)};
       }
     }
     const float ys[2] = {fmaf((float)j, a.d_hi[1], a.lo_hi[1]), fmaf((float)j + 0.5f, a.d_hi[1], a.lo_hi[1])};
@@ -1238,14 +1230,10 @@ __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_consta
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
         F2 E[3], B[3];
-        if constexpr (kGaussZ) {
-          gauss_xy(P, Bz[kOz[c]], xs[kOx[c]], F2(ys[kOy[c]]), E, B);
-        } else {
-          Local<F2> L = Lz[kOz[c]];
-          L.x = xs[kOx[c]];
-          L.y = F2(ys[kOy[c]]);
-          analytic_fields<KIND, AP_FP32_PHASEFF, F2>(P, L, E, B);
-        }
+        Local<F2> L = Lz[kOz[c]];
+        L.x = xs[kOx[c]];
+        L.y = F2(ys[kOy[c]]);
+        analytic_fields<KIND, AP_FP32_PHASEFF, F2>(P, L, E, B);
         v[c] = c < 3 ? E[c] : B[c - 3];
       }
 #pragma unroll
@@ -1484,30 +1472,30 @@ __global__ void __launch_bounds__(256) nodes_plane_kernel(const __grid_constant_
     if (k != kcur) {
       kcur = k;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (!need[h]) continue;
-      const float oz = h ? 0.5f : 0.0f;
-      Pos<PREC> pos;
-      if constexpr (PREC == AP_FP32_PHASEFF) {
-        pos.x = FF{0.0f, 0.0f};
-        pos.y = FF{0.0f, 0.0f};
-        pos.z = node_coord_ff((float)k + oz, a.lo_hi[2], a.lo_lo[2], a.d_hi[2], a.d_lo[2]);
-      } else {
-        pos.load(0.0, 0.0, fma((double)k + oz, a.d[2], a.lo[2]));
+      for (int h = 0; h < 2; ++h) {
+        if (!need[h]) continue;
+        const float oz = h ? 0.5f : 0.0f;
+        Pos<PREC> pos;
+        if constexpr (PREC == AP_FP32_PHASEFF) {
+          pos.x = FF{0.0f, 0.0f};
+          pos.y = FF{0.0f, 0.0f};
+          pos.z = node_coord_ff((float)k + oz, a.lo_hi[2], a.lo_lo[2], a.d_hi[2], a.d_lo[2]);
+        } else {
+          pos.load(0.0, 0.0, fma((double)k + oz, a.d[2], a.lo[2]));
+        }
+        Local<R> L = local_coords<PREC>(P, st, pos);
+        R E[3], B[3];
+        node_values<AP_PLANE, PREC>(P, L, a.current, E, B);
+        if (h == 0) {
+          v[0] = E[0];
+          v[1] = E[1];
+          v[5] = B[2];
+        } else {
+          v[2] = E[2];
+          v[3] = B[0];
+          v[4] = B[1];
+        }
       }
-      Local<R> L = local_coords<PREC>(P, st, pos);
-      R E[3], B[3];
-      node_values<AP_PLANE, PREC>(P, L, a.current, E, B);
-      if (h == 0) {
-        v[0] = E[0];
-        v[1] = E[1];
-        v[5] = B[2];
-      } else {
-        v[2] = E[2];
-        v[3] = B[0];
-        v[4] = B[1];
-      }
-    }
     }
     for (int i = 0; i < a.n_comp; ++i) {
       const int c = a.comp[i];
@@ -1555,9 +1543,9 @@ int launch_nodes_t(const Pulse<Real<PREC>> &P, const NodeArgs &a, void *stream) 
         kern<<<(unsigned)gp, block, 0, s>>>(P, a);
         return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
       }
-      // other beams in float-float arithmetic: two nodes per lane, packed; one
-      // resident wave of blocks, each warp a contiguous run of rows
-      if (!a.current) {
+      // the other beams: two nodes per lane, packed; one resident wave of
+      // blocks, each warp a contiguous run of rows
+      else {
         auto kern = a.f64 ? nodes_row_pair_kernel<KIND, double> : nodes_row_pair_kernel<KIND, float>;
         long long gp = (long long)a.sm_count * occupancy_blocks(kern, block, 0);
         if (gp > (rows + 7) / 8) gp = (rows + 7) / 8;

@@ -149,66 +149,6 @@ using pair::FF2;
 template <>
 struct IsPair<F2> : std::true_type {};
 
-// Positions of the two particles of a thread as float-float pairs, the same
-// compensated accumulation as Pos<AP_FP32_PHASEFF>.  The longitudinal
-// coordinate is held relative to the pulse's focus, dz = z - z_f (formed in
-// double on load), since the carrier phase needs dz to float-float accuracy
-// every step and the absolute z only in float (for the grid).
-struct Pos2 {
-  FF2 x, y, dz;
-  __device__ __forceinline__ void load(const double X[2], const double Y[2], const double Z[2], double zf) {
-    const FF a = split_double(X[0]), b = split_double(X[1]);
-    x = {F2(a.hi, b.hi), F2(a.lo, b.lo)};
-    const FF c = split_double(Y[0]), d = split_double(Y[1]);
-    y = {F2(c.hi, d.hi), F2(c.lo, d.lo)};
-    const FF e = split_double(Z[0] - zf), f = split_double(Z[1] - zf);
-    dz = {F2(e.hi, f.hi), F2(e.lo, f.lo)};
-  }
-  __device__ __forceinline__ static void acc(FF2 &p, F2 d) {
-    const F2 y = d + p.lo;
-    const F2 t = p.hi + y;
-    p.lo = y - (t - p.hi);
-    p.hi = t;
-  }
-  __device__ __forceinline__ void advance(F2 vx, F2 vy, F2 vz, F2 dt_xy, F2 dt) {
-    acc(x, dt_xy * vx);
-    acc(y, dt_xy * vy);
-    acc(dz, dt * vz);
-  }
-  __device__ __forceinline__ F2 xr() const { return x.hi + x.lo; }
-  __device__ __forceinline__ F2 yr() const { return y.hi + y.lo; }
-  // absolute z in float, from z_f = zf_hi + zf_lo
-  __device__ __forceinline__ F2 zr(float zf_hi, float zf_lo) const {
-    return (dz.hi + F2(zf_hi)) + (dz.lo + F2(zf_lo));
-  }
-};
-
-// Local coordinates of both particles at one step (float-float phase), the
-// pairwise form of local_coords<AP_FP32_PHASEFF>: the step's time base `st`
-// is shared by the two particles.
-__device__ __forceinline__ Local<F2> local_coords2(const Pulse<float> &P, const StepFF &st,
-                                                   const Pos2 &pos) {
-  Local<F2> L;
-  const FF2 dz = pos.dz;  // z - z_f
-  // psi = C_n - k dz, k dz = kp + ke with -ke from the negated constant
-  const F2 kp = F2(P.k_hi) * dz.hi;
-  const F2 nke = two_prod_nerr(dz.hi, F2(-P.k_hi), kp);
-  const F2 kdlo = fma(F2(P.k_hi), dz.lo, F2(P.k_lo) * dz.hi) - nke;
-  const FF2 ps = two_diff(F2(st.C), kp);
-  L.psi = reduce_ff(ps.hi, ps.lo - kdlo);
-  L.x = pos.xr();
-  L.y = pos.yr();
-  L.dz = dz.hi + dz.lo;
-  const float Tf = __fadd_rn(st.Th, st.Tl);
-  L.eta = fma(L.dz, F2(-P.inv_vg), F2(Tf));
-  L.T = F2(Tf);
-  // phi' = T - dz as float-float
-  const FF2 ph = two_diff(F2(st.Th), dz.hi);
-  L.phi_hi = ph.hi;
-  L.phi_lo = ph.lo + (F2(st.Tl) - dz.lo);
-  return L;
-}
-
 // The cell test and weights of a thread's two particles with packed
 // arithmetic (grid units, offsets from each cached cell), then each
 // particle's own warp-uniform refetch branch, as grid_fetch does per particle.
