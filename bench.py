@@ -346,20 +346,17 @@ def launch_desc(wl):
 
 NODE_N = 256           # staggered grid edge for the node-evaluation rate
 # FP32 operations of the Gaussian (longitudinal terms on) on the six
-# staggered positions of the nodes: the position part once per component of a
-# node (transverse exponent, angle and its reduction, complex assembly, the one
-# component written: 21).  The z/t part (float-float carrier phase and
-# envelope argument 32, envelope 2, q = 1/(1 - i zeta) 3, for each of the two
-# z levels) is computed once per z index per warp's run of rows: fewer than
-# 0.01 operations per node, not counted.
-NODE_OPS_PER_NODE = 6 * 21
+# staggered positions of the nodes: the separable form's complex products of a
+# column and a row factor (2 per transverse component, 5 per longitudinal one).
+# The factors themselves are made once per column and row of a slab and not
+# counted.
+NODE_OPS_PER_NODE = 18
 NODE_OPS_PER_ROW = 0
 YEE_LINES, YEE_NZ, YEE_STEPS = 152, 8192, 2000
 # 1-D lines with a cold-plasma current (Sec. 4): n_e = 1e-3 n_c, a g = 4
 # super-Gaussian of tau = 30 at 20 cells per wavelength, c dt/dz = 0.9
 LINE_LINES, LINE_NZ, SPLIT_STEPS, PLASMA_STEPS = 304, 4096, 2000, 20000
-SPLIT_MUFU_PER_NODE_STEP = 6  # E1: ex2, sin, cos; J1: ex2 and the sin, cos of its phase shift (its
-                              # carrier is E1's rotated by omega dt/2)
+SPLIT_MUFU_PER_NODE_STEP = 4  # E1: ex2 and cos; J1: ex2 and the sine of its summed phase
 
 
 def closed_form_rate(wl, stream, sum_rate):
