@@ -538,7 +538,8 @@ void default_shape(const ap_handle_s *h, long long n, int precision, bool batche
     if (per_sm >= 1536) a.shape.block = 256;
   } else if (per_sm >= (batched ? 2048 : 640)) {
     a.shape.pairs = 1;
-    a.shape.block = 64;
+    // a large histogram has a copy in each block's shared memory: fewer, larger blocks
+    a.shape.block = a.diag.hist && a.diag.bins > 2048 ? 256 : 64;
   }
 }
 

@@ -107,3 +107,53 @@ def test_step_envelopes_match_oracle(name, env):
     two, _, _ = gpu_push(pulse, parts, -3.0, 0.02, 150, "fp32", launch=dict(block=32, pairs=1))
     _check(one, ref)
     _same(one, two)
+
+
+def _default_and_one(pulse, parts, **kw):
+    args = (pulse, parts, -3.0, 0.02, 12, "fp32")
+    out, dg, st = gpu_push(*args, **kw)
+    one, dg1, _ = gpu_push(*args, launch=dict(block=128), **kw)
+    assert st == 0
+    _same(out, one)
+    return dg, dg1
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("grid,per_sm", [(False, 640), (True, 1536)])
+def test_default_shape_gives_the_same_bits_on_both_sides_of_its_lines(grid, per_sm):
+    """The library's own launch shape (no ap_set_launch) just below and just
+    above the sizes where it changes, against one particle per thread."""
+    import torch
+    from paper_2307_04843_gb300 import _lib
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    pulse = dict(BASE, pol="x", **KINDS["gauss"])
+    g = None
+    if grid:
+        box = ((-4 * L, 4 * L),) * 2 + ((-5 * L, 5 * L),)
+        f = torch.as_tensor(workloads.grid_field(box, 20, amplitude=0.2)).cuda()
+        g = _lib.pack_grid((f, tuple(b[0] for b in box), tuple(b[1] for b in box)), layout="cells")
+    for n in (per_sm * sms - 1, per_sm * sms + 1):
+        dg, dg1 = _default_and_one(pulse, _parts(n), grid=g, hist=(4096, 0.0, 20.0))
+        np.testing.assert_array_equal(dg["hist"], dg1["hist"])
+
+
+@pytest.mark.gpu
+def test_default_shape_batched():
+    import torch
+    from paper_2307_04843_gb300 import _lib
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    pulses = [dict(BASE, pol=p, **KINDS["gauss"]) for p in ("x", "cm", "y")]
+    for n in (2048 * sms - 1, 2048 * sms + 1):
+        parts = _parts(n)
+        off = torch.tensor([0, n // 5, n // 5, n], dtype=torch.int64, device="cuda")
+        res = []
+        for launch in (None, dict(block=128)):
+            with _lib.Handle(pulses) as h:
+                if launch:
+                    h.set_launch(**launch)
+                dev = _lib.to_device(parts, "fp32")
+                ws = torch.zeros(64, dtype=torch.int32, device="cuda")
+                _lib.ap_gather_push_batched(h.h, dev, off, None, -3.0, 0.02, 12, "fp32", None, ws)
+                assert h.status() == 0
+                res.append(_lib.to_host(dev))
+        _same(*res)
