@@ -152,18 +152,17 @@ struct IsPair<F2> : std::true_type {};
 // The cell test and weights of a thread's two particles with packed
 // arithmetic (grid units, offsets from each cached cell), then each
 // particle's own warp-uniform refetch branch, as grid_fetch does per particle.
-// gk: the factors and offsets from the coordinates (x, y, and z in the step's
-// own units) to grid units, pre-broadcast in shared memory,
-// gk[a] = (factor, factor, offset, offset), and gk[3] = (1/2, 1/2, -, -):
+// fz: the grid unit along z.
+// gk: the factors and offsets from x and y to grid units, pre-broadcast in
+// shared memory, gk[a] = (factor, factor, offset, offset), and gk[3] = (1/2, 1/2, -, -):
 // a 16-byte load yields both pair operands, where constants kept in the
 // kernel parameters would be re-broadcast into register pairs every step
 // (the two-particle kernels run at their register limit).
 template <class CA, class CB>
-__device__ __forceinline__ void grid_fetch2(const GridView &g, CA &ga, CB &gb, F2 x, F2 y, F2 z,
+__device__ __forceinline__ void grid_fetch2(const GridView &g, CA &ga, CB &gb, F2 x, F2 y, F2 fz,
                                             const float4 *gk) {
-  const float4 kx = gk[0], ky = gk[1], kz = gk[2], kh = gk[3];
-  F2 f[3] = {fma(x, F2(kx.x, kx.y), F2(kx.z, kx.w)), fma(y, F2(ky.x, ky.y), F2(ky.z, ky.w)),
-             fma(z, F2(kz.x, kz.y), F2(kz.z, kz.w))};
+  const float4 kx = gk[0], ky = gk[1], kh = gk[3];
+  F2 f[3] = {fma(x, F2(kx.x, kx.y), F2(kx.z, kx.w)), fma(y, F2(ky.x, ky.y), F2(ky.z, ky.w)), fz};
 #pragma unroll
   for (int a = 0; a < 3; ++a)
     f[a] = F2(fminf(fmaxf(f[a].x, 0.0f), g.top[a]), fminf(fmaxf(f[a].y, 0.0f), g.top[a]));

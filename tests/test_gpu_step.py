@@ -157,3 +157,37 @@ def test_default_shape_batched():
                 assert h.status() == 0
                 res.append(_lib.to_host(dev))
         _same(*res)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("z_focus", [2 * math.pi * 1e3, -2 * math.pi * 1e4])
+def test_grid_gather_with_the_focus_far_from_the_grid(z_focus):
+    """The grid unit along z is good to 2^-24 of itself wherever the pulse's
+    focus (the origin of the step's longitudinal coordinate) lies.
+
+    Node values of size A = 0.5 without any smoothness: a weight error of e
+    cells in each of three directions moves the field by up to 6 A e.  With 33
+    nodes e <= 3 * 2^-24 * 32, so over a time of 3 the momentum moves by
+    5e-5, about 1e-4 with what the trajectory feeds back.  An error of 2^-24 of
+    the focus distance in cells would move it by 1e-3 and 1e-2."""
+    import torch
+    from paper_2307_04843_gb300 import _lib
+    rng = np.random.default_rng(7)
+    box = ((-16.0, 16.0),) * 3
+    lo, hi = (-16.0,) * 3, (16.0,) * 3
+    g = np.float32(rng.uniform(-0.5, 0.5, (6, 33, 33, 33)))
+    parts = workloads.particles_uniform(box, 257, 3)
+    pulse = dict(kind="gauss", pol="x", env="gauss", env_len=25.0, a0=0.0, omega=1.0, w0=10.0, z_focus=z_focus)
+    args = (pulse, parts, 0.3, 0.05, 60, "fp32")
+    ref = oracle.push(pulse, parts, 0.3, 0.05, 60, grid=(g, lo, hi), threads=THREADS)
+    dev = torch.as_tensor(g).cuda()
+    cells = _lib.pack_grid((dev, lo, hi), layout="cells")
+    outs = [gpu_push(*args, grid=cells, launch=kw)[0]
+            for kw in (dict(block=64), dict(block=64, grid_cache=1), dict(block=64, pairs=1),
+                       dict(block=64, pairs=1, grid_cache=1), dict(block=64, pairs=1, grid_cache=2))]
+    arrays = gpu_push(*args, grid=(dev, lo, hi), launch=dict(block=64))[0]
+    for out in outs[:1] + [arrays]:
+        d = max(np.max(np.abs(out[k] - ref[k])) for k in ("ux", "uy", "uz"))
+        assert d <= 1e-4, d
+    for out in outs[1:]:
+        _same(outs[0], out)
