@@ -368,12 +368,17 @@ void derive(const ap_pulse_desc &d, Pulse<double> &P, Pulse<float> &F) {
   S.circ = d.pol == AP_CIRC_P || d.pol == AP_CIRC_M ? 1 : 0;
   const double senv = P.env == AP_ENV_GAUSS ? std::sqrt(P.env_a)
                       : P.env == AP_ENV_SIN2 || P.env == AP_ENV_SGAUSS ? P.env_a : 1.0;
-  S.s_env = (float)senv;
   S.env_len = (float)(1.0 / senv);
   S.env_w = (float)(P.env_a * P.env_b);
+  // The factor of Z is rounded to float; the factor of T is what belongs to the
+  // rounded one, in two floats.  Two factors rounded each for itself would leave
+  // 2^-24 (t - t_f) of eta where the two terms cancel; this one scales eta as a
+  // whole by 1 + 2^-25 at most.
   S.c_eta = (float)(-senv * P.inv_vg * S.z_len);
+  const double sT = -(double)S.c_eta / (P.inv_vg * S.z_len);
+  split(std::isfinite(sT) ? sT : senv, S.s_env, S.s_env_lo);
   S.c_zn = (float)(-P.inv_zR * S.z_len);
-  S.c_tz = (float)(P.beta_f * P.inv_zR);
+  split(-(double)S.c_zn * P.beta_f / S.z_len, S.c_tz, S.c_tz_lo);
   S.c_a = (float)(P.inv_w0sq * log2e);
   double A = P.amp, ce = P.lonE * -2.0 * P.inv_w0sq, cb = P.lonB * -2.0 * P.inv_w0sq;
   if (d.kind == AP_LG) {

@@ -33,9 +33,12 @@ struct Comp {
 struct FastPulse {
   double z_scale, z_len;  // k / 2 pi and 2 pi / k
   double turn0;           // carrier phase that the frame adds (turns)
-  float s_env, env_len;   // scale of the envelope argument, and its inverse
+  float s_env, s_env_lo, env_len;  // scale of the envelope argument (hi, lo), and its inverse
   float env_w;            // half-width of the sin^2 window, scaled
-  float c_eta, c_zn, c_tz;  // eta s_env = s_env T + c_eta Z, -zeta = c_zn Z + c_tz T
+  // eta s_env = s_env T + c_eta Z, -zeta = c_zn Z + c_tz T; the factors of T
+  // (hi, lo) are made from the rounded factors of Z, so that the two terms
+  // cancel exactly far from the focus
+  float c_eta, c_zn, c_tz, c_tz_lo;
   float c_a;              // log2(e) / w0^2
   float A, Abr, Ace, Acb;  // E_perp, B_perp, E_z, B_z per unit field
   float lg_n[6][kLgMaxP];  // the Laguerre recurrences with the subtracted terms' signs in

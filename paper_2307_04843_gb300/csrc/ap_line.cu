@@ -301,6 +301,10 @@ int launch_split(const SplitArgs &sa, void *stream) {
 
 SplitArgs split_args(const Pulse<double> &pd, const Pulse<float> &pf, const LineArgs &a) {
   SplitArgs s;
+  auto split = [](double v, float &hi, float &lo) {
+    hi = (float)v;
+    lo = (float)(v - (double)hi);
+  };
   s.line = a;
   s.fast = pf.fast;
   s.env = pd.env;
@@ -320,19 +324,16 @@ SplitArgs split_args(const Pulse<double> &pd, const Pulse<float> &pf, const Line
   } else if (pd.env == AP_ENV_SIN2) {
     su = pd.env_a;
   }
-  s.fast.s_env = (float)su;
-  s.fast.c_tz = 0.0f;
+  // the scale of t - t_f from the rounded one of z - z_f (see FastPulse)
+  s.su_vg = (float)(su * pd.inv_vg);
+  split((double)s.su_vg / pd.inv_vg, s.fast.s_env, s.fast.s_env_lo);
+  s.fast.c_tz = s.fast.c_tz_lo = 0.0f;
   GridView none;
   std::memset(&none, 0, sizeof(none));
   s.base = make_step_base(pf, a.t0, a.dt, none);
-  auto split = [](double v, float &hi, float &lo) {
-    hi = (float)v;
-    lo = (float)(v - (double)hi);
-  };
   split(pf.fast.z_scale, s.zs_hi, s.zs_lo);
   s.zf_hi = pf.zf_hi;
   s.zf_lo = pf.zf_lo;
-  s.su_vg = (float)(su * pd.inv_vg);
   s.hu = (float)(0.5 * a.dt * su);
   s.env_w = (float)(pd.env_a * pd.env_b);
   s.amp = (float)pd.amp;

@@ -189,8 +189,10 @@ __device__ __forceinline__ float4 step_entry(const FastPulse &F, const StepBase 
     const FF c = two_sum(s.om0.hi, nd.hi);
     const float clo = __fadd_rn(__fadd_rn(c.lo, nd.lo), __fmaf_rn(nf, s.del.lo, s.om0.lo));
     const float C = __fadd_rn(__fsub_rn(c.hi, round_magic(c.hi)), clo);
-    return make_float4(C, __fmaf_rn(T.hi, F.s_env, __fmul_rn(T.lo, F.s_env)),
-                       __fmaf_rn(T.hi, F.c_tz, __fmul_rn(T.lo, F.c_tz)), __fadd_rn(T.hi, T.lo));
+    auto scaled = [&](float hi, float lo) {  // (hi + lo) T
+      return __fmaf_rn(T.hi, hi, __fmaf_rn(T.hi, lo, __fmul_rn(T.lo, hi)));
+    };
+    return make_float4(C, scaled(F.s_env, F.s_env_lo), scaled(F.c_tz, F.c_tz_lo), __fadd_rn(T.hi, T.lo));
   }
 }
 

@@ -191,3 +191,30 @@ def test_grid_gather_with_the_focus_far_from_the_grid(z_focus):
         assert d <= 1e-4, d
     for out in outs[1:]:
         _same(outs[0], out)
+
+
+@pytest.mark.gpu
+def test_envelope_argument_far_from_the_focus():
+    """eta = (t - t_f) - (z - z_f)/v_g of an electron that meets the pulse at a
+    large distance D = 1.04e6 from the focus is good to the rounding of t - t_f
+    and of z - z_f.  The first is the same for all particles of a step, at most
+    2^-25 2^20 = 0.031 here; the second averages out over 4000 particles (0.03 /
+    sqrt(4000)), so the mean error stays within 0.035.  A mismatch between the
+    factors of the two terms would add up to 2^-24 D = 0.06 to it, and 0.099 for
+    this envelope if each factor is rounded to float for itself."""
+    D, T = 1.04e6, 22.5
+    rng = np.random.default_rng(11)
+    n = 4000
+    eta = rng.uniform(8.0, 14.0, n)
+    eta = eta[np.cos(eta) > 0.5]
+    n = eta.size
+    zero = np.zeros(n)
+    parts = dict(x=zero.copy(), y=zero.copy(), z=D - eta, ux=zero.copy(), uy=zero.copy(), uz=zero.copy())
+    pulse = dict(kind="plane", pol="x", env="gauss", env_len=T, a0=1.0, omega=1.0)
+    ref = oracle.push(pulse, parts, D, 1e-3, 1, threads=THREADS)
+    for launch in (dict(block=32), dict(block=32, pairs=1)):
+        out, _, st = gpu_push(pulse, parts, D, 1e-3, 1, "fp32", launch=launch)
+        assert st == 0
+        # d ln Gamma = -4 ln2 eta / T^2 d eta
+        d = -np.log(out["ux"] / ref["ux"]) * T * T / (4 * math.log(2.0) * eta)
+        assert abs(np.mean(d)) <= 0.035, np.mean(d)
