@@ -50,7 +50,7 @@ template <typename R, int NT>
 struct PulseAD {
   static constexpr bool kHasPlasma = true;
   int32_t kind, pol, env, lon, lg_p, lg_al, lg_sgn, sg_order, plasma;
-  R amp, bratio, lonE, lonB, env_a, env_b, px_re, px_im, py_re, py_im;
+  R amp, bratio, lonE, lonB, env_a, env_b, sg_max, px_re, px_im, py_re, py_im;
   R fdc, inv_w, lg_c1, lg_c2;  // plane wave in a plasma (Sec. 4, Eq. b_corr_t)
   R lg_alf;                    // |l| as a number
   R lg_r[6][kLgMaxP];
@@ -67,7 +67,7 @@ __device__ __forceinline__ PulseAD<R, NT> make_ad(const Pulse<R> &P) {
   A.lg_alf = P.lg_alf;
   A.amp = P.amp_unit;  // unit a0: the physical field is a0 times this one
   A.bratio = P.bratio; A.lonE = P.lonE; A.lonB = P.lonB;
-  A.env_a = P.env_a; A.env_b = P.env_b;
+  A.env_a = P.env_a; A.env_b = P.env_b; A.sg_max = P.sg_max;
   A.px_re = P.px_re; A.px_im = P.px_im; A.py_re = P.py_re; A.py_im = P.py_im;
   for (int r = 0; r < 6; ++r)
     for (int k = 0; k < kLgMaxP; ++k) A.lg_r[r][k] = P.lg_r[r][k];
@@ -213,7 +213,7 @@ __device__ __forceinline__ R envelope_dlog(const PT &P, R eta, R mul) {
     case AP_ENV_GAUSS:
       return R(-2 * kLn2) * P.env_a * eta;
     case AP_ENV_SGAUSS: {
-      const R u = eta * P.env_a;
+      const R u = sg_bound(eta * P.env_a, P.sg_max);
       const R s = u * u;
       R p = R(1);  // s^(g-1)
       for (int i = 1; i < P.sg_order; ++i) p *= s;
@@ -726,10 +726,10 @@ __device__ __forceinline__ F2 dlog_scaled(const PT &P, F2 e, F2 mul) {
     case AP_ENV_GAUSS:
       return F2(-1.38629436f * P.fast.s_env) * e;
     case AP_ENV_SGAUSS: {
-      const F2 s = e * e;
+      const F2 u = sg_bound(e, P.sg_max), s = u * u;
       F2 p = F2(1.0f);
       for (int i = 1; i < P.sg_order; ++i) p *= s;
-      return F2(-1.38629436f * P.env_b * (float)P.sg_order * P.fast.s_env) * e * p;
+      return F2(-1.38629436f * P.env_b * (float)P.sg_order * P.fast.s_env) * u * p;
     }
     default:
       return F2(0.0f);

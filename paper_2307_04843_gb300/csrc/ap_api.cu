@@ -241,6 +241,7 @@ void derive(const ap_pulse_desc &d, Pulse<double> &P, Pulse<float> &F) {
     case AP_ENV_SGAUSS:
       P.env_a = 1.0 / d.env_len;
       P.env_b = 1.4426950408889634;
+      P.sg_max = std::pow(760.0, 0.5 / d.sg_order);  // e^-760 < 2^-1096
       break;
     default:
       break;
@@ -330,6 +331,7 @@ void derive(const ap_pulse_desc &d, Pulse<double> &P, Pulse<float> &F) {
   F.lonE = (float)P.lonE; F.lonB = (float)P.lonB;
   F.inv_w0sq = (float)P.inv_w0sq; F.inv_zR = (float)P.inv_zR;
   F.env_a = (float)P.env_a; F.env_b = (float)P.env_b;
+  F.sg_max = P.env == AP_ENV_SGAUSS ? (float)std::pow(110.0, 0.5 / d.sg_order) : 0.0f;  // e^-110 < 2^-158
   F.px_re = (float)P.px_re; F.px_im = (float)P.px_im;
   F.py_re = (float)P.py_re; F.py_im = (float)P.py_im;
   for (int r = 0; r < 6; ++r)

@@ -351,6 +351,17 @@ __device__ __forceinline__ Local<Real<PREC>> local_coords(const PulseHead<Real<P
 }
 
 // ------------------------------------------------------------ envelope
+// The derivatives of a super-Gaussian grow like u^(2g - 1) and its square where
+// the envelope itself is zero, and overflow from u = 4 (order 16, float) or u =
+// 23 (order 8) on: zero times infinity.  What is multiplied by the envelope is
+// therefore formed from u held within the argument at which the envelope
+// underflows to zero (the same bits inside, finite outside).
+__device__ __forceinline__ float sg_bound(float u, float m) { return fminf(fmaxf(u, -m), m); }
+__device__ __forceinline__ double sg_bound(double u, double m) { return fmin(fmax(u, -m), m); }
+// only where the envelope's own power is differentiated (dual numbers)
+__device__ __forceinline__ float sg_bound_ad(float u, float) { return u; }
+__device__ __forceinline__ double sg_bound_ad(double u, double) { return u; }
+
 // Gamma(eta) split into a multiplicative factor `mul` and an additive
 // base-2 exponent `l2` (Gaussian and super-Gaussian envelopes share the
 // beam's exp2).  SIN2: env_a = pi/T, env_b = T/2; GAUSS: env_a = 2 ln2 log2e
@@ -377,7 +388,7 @@ __device__ __forceinline__ void envelope(const PT &P, R eta, R &mul, R &l2) {
       l2 = -P.env_a * eta * eta;
       break;
     case AP_ENV_SGAUSS: {
-      R s = eta * P.env_a;
+      R s = sg_bound_ad(eta * P.env_a, P.sg_max);
       s = s * s;
       R p = s;
       for (int i = 1; i < P.sg_order; ++i) p *= s;
@@ -471,7 +482,7 @@ __device__ __forceinline__ void envelope_logd(const PT &P, R eta, R &L1, R &L2) 
     L1 = -P.lg_c1 * eta;
     L2 = L1 * L1 - P.lg_c2;
   } else if (P.env == AP_ENV_SGAUSS) {
-    const R u = eta * P.env_a;
+    const R u = sg_bound(eta * P.env_a, P.sg_max);
     const R s = u * u;
     R q = R(1);
     for (int i = 1; i < P.sg_order; ++i) q *= s;

@@ -153,6 +153,18 @@ template <typename R, int N>
 __device__ __forceinline__ Dual<R, N> fabs(const Dual<R, N> &a) {
   return a.v < R(0) ? -a : a;
 }
+// the value held within the bound, the tangents kept: they then meet the
+// exponential's zero as finite numbers
+template <typename R, int N>
+__device__ __forceinline__ Dual<R, N> sg_bound(Dual<R, N> u, R m) {
+  u.v = sg_bound(u.v, m);
+  return u;
+}
+template <typename R, int N>
+__device__ __forceinline__ Dual<R, N> sg_bound_ad(Dual<R, N> u, R m) {
+  return sg_bound(u, m);
+}
+
 template <typename R, int N>
 __device__ __forceinline__ Dual<R, N> rcp_r(const Dual<R, N> &a) {
   Dual<R, N> r;

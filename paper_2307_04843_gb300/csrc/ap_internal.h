@@ -64,6 +64,7 @@ struct PulseHead {
   R inv_w0sq;       // 1 / w0^2
   R inv_zR;         // 1 / z_R
   R env_a, env_b;   // envelope constants (see ap_device.cuh)
+  R sg_max;         // |eta/tau| from which a super-Gaussian is exactly zero in R (see sg_bound)
   R px_re, px_im, py_re, py_im;  // polarisation vector p
   // Laguerre three-term recurrence (k+1) L_{k+1} = (2k+1+a-s) L_k - (k+a) L_{k-1}
   // as L_{k+1} = (lg_r[0][k] - lg_r[1][k] s) L_k - lg_r[2][k] L_{k-1}, for

@@ -23,6 +23,7 @@
 // loop of the same expressions bit for bit.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -134,6 +135,8 @@ struct SplitArgs {
   float zf_hi, zf_lo;
   float su_vg;              // scale of the envelope argument over v_g
   float hu;                 // dt/2 in the scaled argument
+  bool finite;              // th and A stay finite over all nodes and steps of the call
+  float s_max;              // square of the scaled argument from which the super-Gaussian is zero
   float env_w;              // half-width of the sin^2 window, scaled
   float amp, jamp;          // a0, and the amplitude of J1
   float delta;              // omega dt/2
@@ -248,12 +251,15 @@ __global__ void __launch_bounds__(MAXT) split_line_kernel(const __grid_constant_
         m1 = window2(u1, sa.env_w);
       } else {
         m0 = exp2_neg(upow<G>(rmul(u0, u0), sa.g));
-        const F2 s = rmul(u1, u1);
         if constexpr (G == 1) {
-          m1 = exp2_neg(s);
+          m1 = exp2_neg(rmul(u1, u1));
           th = rmul(F2(sa.k1), u1);
           A = rfma(rmul(F2(-0.5f), th), th, F2(1.0f + sa.k2));
         } else {
+          F2 s = rmul(u1, u1);
+          // held where the envelope is zero, as th and A would overflow (see
+          // sg_bound; the compiled orders are for lines on which they do not)
+          if constexpr (G == kOrderAny) s = F2(fminf(s.x, sa.s_max), fminf(s.y, sa.s_max));
           F2 q = F2(1.0f);
           if (G > 1 || sa.g > 1) q = upow<(G > 1 ? G - 1 : 0)>(s, sa.g - 1);
           m1 = exp2_neg(rmul(q, s));
@@ -295,7 +301,7 @@ template <int C, int MAXT>
 int launch_split(const SplitArgs &sa, void *stream) {
   if (sa.env == AP_ENV_SIN2) return launch_split_g<C, MAXT, kSin2>(sa, stream);
   if (sa.g == 1) return launch_split_g<C, MAXT, 1>(sa, stream);
-  if (sa.g == 4) return launch_split_g<C, MAXT, 4>(sa, stream);
+  if (sa.g == 4 && sa.finite) return launch_split_g<C, MAXT, 4>(sa, stream);
   return launch_split_g<C, MAXT, kOrderAny>(sa, stream);
 }
 
@@ -335,6 +341,7 @@ SplitArgs split_args(const Pulse<double> &pd, const Pulse<float> &pf, const Line
   s.zf_hi = pf.zf_hi;
   s.zf_lo = pf.zf_lo;
   s.hu = (float)(0.5 * a.dt * su);
+  s.s_max = (float)std::pow(158.0, 1.0 / s.g);  // 2^-158 is zero in float
   s.env_w = (float)(pd.env_a * pd.env_b);
   s.amp = (float)pd.amp;
   s.jamp = (float)(pd.jamp * pd.amp);
@@ -342,6 +349,11 @@ SplitArgs split_args(const Pulse<double> &pd, const Pulse<float> &pf, const Line
   s.k1 = (float)(-pd.lg_c1 * pd.inv_w * std::pow(ratio, 2.0 * s.g - 1.0));
   s.k2 = (float)(pd.lg_c2 * pd.inv_w * pd.inv_w * std::pow(ratio, 2.0 * s.g - 2.0));
   if (pd.env != AP_ENV_GAUSS && pd.env != AP_ENV_SGAUSS) s.k1 = s.k2 = 0.0f;
+  // largest |u| of the call: either end of the line at either end of the time
+  const double T = std::max(std::fabs(a.t0 - pd.t_f), std::fabs(a.t0 + ((double)a.n_steps + 1.0) * a.dt - pd.t_f));
+  const double Z = std::max(std::fabs(a.z0 - pd.z_f), std::fabs(a.z0 + (double)a.nz * a.dz - pd.z_f));
+  const double u = std::max(1.0, su * (T + Z * pd.inv_vg)), q = std::pow(u, 2.0 * s.g - 2.0);
+  s.finite = std::fabs(s.k1) * u * q < 1e18 && std::fabs(s.k2) * q < 1e36;  // A takes in th^2
   return s;
 }
 

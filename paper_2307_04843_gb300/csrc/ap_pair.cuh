@@ -85,6 +85,11 @@ __device__ __forceinline__ F2 sin2_window(F2 m, F2 eta, float b) {
   return F2(fabsf(eta.x) > b ? 0.0f : m.x, fabsf(eta.y) > b ? 0.0f : m.y);
 }
 
+__device__ __forceinline__ F2 sg_bound(F2 u, float m) {
+  return F2(fminf(fmaxf(u.x, -m), m), fminf(fmaxf(u.y, -m), m));
+}
+__device__ __forceinline__ F2 sg_bound_ad(F2 u, float) { return u; }
+
 // complex product with two fused operations per part
 __device__ __forceinline__ Cx<F2> cmul(Cx<F2> a, Cx<F2> b) {
   return {fma(a.re, b.re, -(a.im * b.im)), fma(a.re, b.im, a.im * b.re)};
