@@ -18,9 +18,9 @@
 namespace apt {
 
 // A packed product that stays apart from the sum it feeds: the assembler fuses
-// a packed multiplication with the packed addition that follows it, whatever
-// rounding the two are written with, while the lines have to reproduce a plain
-// loop of separately rounded operations bit for bit.  a b + (-0) is the rounded
+// a packed multiplication whose only uses are sums with each of them (see
+// ap_pair.cuh), while the lines have to reproduce a plain loop of separately
+// rounded operations bit for bit.  a b + (-0) is the rounded
 // product, signs of zeros included, in one operation that nothing can be fused
 // into; the -0 comes as a kernel argument, so that it is not known to be one.
 struct LineMul {

@@ -13,9 +13,12 @@
 // operations stay one per particle.
 //
 // Every packed operation rounds each half exactly as the scalar _rn
-// intrinsic does (round to nearest even, no contraction), so the error-free
-// transformations of the float-float phase and position carry over
-// unchanged.
+// intrinsic does (round to nearest even), with one exception: a product whose
+// only uses are sums is fused with each of them by the assembler, whatever
+// rounding the two are written with (measured: a + b c, a - b c and two sums of
+// one product come out fused, a product that is also stored or multiplied
+// on does not).  The products of the error-free transformations also enter a
+// fused operation, so those carry over unchanged.
 #pragma once
 
 #include "ap_device.cuh"

@@ -25,8 +25,9 @@
 //
 // For a linearly polarised Gaussian beam this is 77 packed operations per
 // step against 131.  Every operation is written with a single rounding
-// (rmul, radd, rsub, rfma), so the one- and two-particle kernels give the
-// same bits.
+// (rmul, radd, rsub, rfma), and no product has sums alone for its uses (the
+// assembler would fuse a packed one with them, see ap_pair.cuh), so the one- and
+// two-particle kernels give the same bits.
 //
 // Measured on a GB300, before and after (two particles per thread; ncu of the
 // batched Gaussian: 112 instructions per pair-step, FMA pipe 71 %, special
@@ -278,12 +279,26 @@ __device__ __forceinline__ UnitFields<R> unit_fields_beam(const PT &P, const flo
     o.Vr = o.Ur;
     o.Vi = o.Ui;
     if (P.plasma) {
+      // B from the finite-duration terms (envelope_logd and finite_duration, in
+      // operations of one rounding)
       const R e = rmul(eta, R(F.env_len));  // back to the envelope's own argument
-      R L1, L2;
-      envelope_logd(P, e, L1, L2);
-      const Cx<R> V = finite_duration(Cx<R>{o.Ur, o.Ui}, P.fdc, L1, L2, P.inv_w);
-      o.Vr = V.re;
-      o.Vi = V.im;
+      R L1 = R(0.0f), L2 = R(0.0f);
+      if (P.env == AP_ENV_GAUSS) {
+        L1 = rmul(R(-P.lg_c1), e);
+        L2 = rfma(L1, L1, R(-P.lg_c2));
+      } else if (P.env == AP_ENV_SGAUSS) {
+        const R u = sg_bound(rmul(e, R(P.env_a)), P.sg_max), s2 = rmul(u, u);
+        R q = R(1.0f);
+        for (int i = 1; i < P.sg_order; ++i) q = rmul(q, s2);
+        L1 = rmul(rmul(R(-P.lg_c1), u), q);
+        L2 = rfma(L1, L1, rmul(R(-P.lg_c2), q));
+      }
+      const R th = rmul(rmul(R(P.fdc), L1), R(P.inv_w));
+      const R A = rfma(rmul(R(0.5f), th), th, rfma(rmul(rmul(R(-P.fdc), L2), R(P.inv_w)), R(P.inv_w), R(1.0f)));
+      R sn_t, cs_t;
+      sincos_r(th, &sn_t, &cs_t);
+      o.Vr = rmul(A, rfma(o.Ur, cs_t, rmul(rneg(o.Ui), sn_t)));
+      o.Vi = rmul(A, rfma(o.Ur, sn_t, rmul(o.Ui, cs_t)));
     }
     o.ez = R(0.0f);
     o.bz = R(0.0f);
@@ -317,7 +332,7 @@ __device__ __forceinline__ UnitFields<R> unit_fields_beam(const PT &P, const flo
       // u = (x + i sgn y)^l L_p^l(s) q^{l+1} (q/q*)^p e^{-r^2 q / w0^2}, l = |l|,
       // s = 2 r^2 |q|^2 / w0^2, (sqrt2 / w0)^l inside the amplitude factor
       const R bi = rmul(b, inv);
-      R mag = exp2_neg(radd(bi, g));
+      R mag = exp2_neg(rfma(b, inv, g));
       if constexpr (ENV == kEnvAny) mag = rmul(mag, mul);
       const R s = rmul(bi, R(1.38629436f));  // 2 / log2(e)
       const Cx<R> q{inv, qi};
@@ -329,7 +344,7 @@ __device__ __forceinline__ UnitFields<R> unit_fields_beam(const PT &P, const flo
       for (int i = 0; i < P.lg_al; ++i) K = rcmul(K, q, nq);
       if (P.lg_p > 0) {
         const Cx<R> gg{rfma(R(2.0f), inv, R(-1.0f)), radd(qi, qi)};
-        const R ngi = radd(nq, nq);
+        const R ngi = rmul(R(2.0f), nq);
         K = rcmul(K, gg, ngi);
         Lp = rfma(R(F.lg_n[1][0]), s, R(F.lg_n[0][0]));
         nD = R(1.0f);

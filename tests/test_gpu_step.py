@@ -218,3 +218,29 @@ def test_envelope_argument_far_from_the_focus():
         # d ln Gamma = -4 ln2 eta / T^2 d eta
         d = -np.log(out["ux"] / ref["ux"]) * T * T / (4 * math.log(2.0) * eta)
         assert abs(np.mean(d)) <= 0.035, np.mean(d)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("pol", ["x", "y", "cp", "cm"])
+@pytest.mark.parametrize("env", [dict(env="gauss", env_len=15.0), dict(env="sgauss", sg_order=1, env_len=9.0),
+                                 dict(env="sgauss", sg_order=5, env_len=12.0), dict(env="cw")])
+def test_plasma_pulse_gives_the_same_bits_in_every_shape(env, pol):
+    """The finite-duration terms of a pulse in a plasma round alike with one and
+    two particles per thread, without a grid and with every cell cache."""
+    import torch
+    from paper_2307_04843_gb300 import _lib
+    pulse = dict(kind="plane", pol=pol, a0=2.0, omega=1.0, omega_p=0.4, phase0=0.3, z_focus=0.7, **env)
+    parts = _parts(199)
+    box = ((-4 * L, 4 * L),) * 2 + ((-5 * L, 5 * L),)
+    lo, hi = tuple(b[0] for b in box), tuple(b[1] for b in box)
+    g = workloads.grid_field(box, 20, amplitude=0.2)
+    cells = _lib.pack_grid((torch.as_tensor(g).cuda(), lo, hi), layout="cells")
+    args = (pulse, parts, -3.0, 0.02, 150, "fp32")
+    one, _, st = gpu_push(*args, launch=dict(block=32))
+    assert st == 0
+    _check(one, oracle.push(pulse, parts, -3.0, 0.02, 150, threads=THREADS))
+    _same(one, gpu_push(*args, launch=dict(block=32, pairs=1))[0])
+    base, _, _ = gpu_push(*args, grid=cells, launch=dict(block=64))
+    for launch in (dict(block=64, grid_cache=1), dict(block=64, pairs=1), dict(block=64, pairs=1, grid_cache=1),
+                   dict(block=64, pairs=1, grid_cache=2)):
+        _same(base, gpu_push(*args, grid=cells, launch=launch)[0])
