@@ -961,13 +961,11 @@ inline size_t push_smem_head(int block) {
   return step_table_bytes(block) + grid_cache_bytes<PREC, GRID, NP>(block);
 }
 
+// opt in above what every kernel gets without asking: 48 KB less its static
+// shared memory (up to 14 KB here: a pulse, a component table)
 template <typename K>
 inline int set_smem(K kern, size_t smem) {
-  if (smem <= 48 * 1024) return AP_OK;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-                 cudaSuccess
-             ? AP_OK
-             : AP_ERR_CUDA;
+  return smem <= 32 * 1024 ? AP_OK : allow_smem(reinterpret_cast<const void *>(kern));
 }
 
 template <int KIND, int PREC, int GRID>

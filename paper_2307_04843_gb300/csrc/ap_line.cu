@@ -291,8 +291,7 @@ int launch_split_g(const SplitArgs &sa, void *stream) {
   auto kern = split_line_kernel<C, MAXT, G>;
   const int block = line_block<C>(sa.line.nz);
   const size_t smem = 3 * sizeof(F2) * (size_t)C * block;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return AP_ERR_CUDA;
+  if (set_smem(kern, smem) != AP_OK) return AP_ERR_CUDA;
   kern<<<(unsigned)sa.line.n_lines, block, smem, static_cast<cudaStream_t>(stream)>>>(sa);
   return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
 }
@@ -361,8 +360,7 @@ template <typename T, bool APT>
 int launch_line_t(const Pulse<double> &P, const LineArgs &a, void *stream) {
   auto kern = line_kernel<T, APT>;
   const size_t smem = 4u * sizeof(T) * (size_t)a.nz;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return AP_ERR_CUDA;
+  if (set_smem(kern, smem) != AP_OK) return AP_ERR_CUDA;
   int block = (a.nz + 31) / 32 * 32;
   if (block > kLineBlock) block = kLineBlock;
   kern<<<(unsigned)a.n_lines, block, smem, static_cast<cudaStream_t>(stream)>>>(P, a);
