@@ -535,14 +535,20 @@ int default_block(const ap_handle_s *h, long long n, int precision) {
 //     157 / 146 us, Gaussian 1e5 118 / 115, 1e6 376 / 361, 3e6 992 / 915; below,
 //     one is as fast or faster: LG 1e4 115 / 119);
 //   - batched, no grid: two from 2048 per SM (256 sets, 6e5 311 / 285 us; 64
-//     sets, 2e5 174 / 183).
+//     sets, 2e5 174 / 183);
+//   - batched, per-cell coefficients: one, its cell in registers, in blocks of
+//     64, since the block is also the tile that each set is padded to (50 steps,
+//     sets x particles, blocks of 64 / 128 / 256: 4000 x 60 230 / 286 / 456 us,
+//     4000 x 130 425 / 450 / 466, 4000 x 200 527 / 459 / 483, 2000 x 1000
+//     758 / 774 / 820, 64 x 20000 466 / 477 / 516, 256 x 8000 726 / 748 / 810).
 void default_shape(const ap_handle_s *h, long long n, int precision, bool batched, apt::PushArgs &a) {
   if (h->shape_set || precision != AP_FP32_PHASEFF) return;
   const long long per_sm = n / (h->sm_count > 0 ? h->sm_count : 1);
   if (a.grid_on) {
     if (!a.grid.cells) return;
     a.shape.grid_cache = 1;
-    if (per_sm >= 1536) a.shape.block = 256;
+    if (batched) a.shape.block = 64;
+    else if (per_sm >= 1536) a.shape.block = 256;
   } else if (per_sm >= (batched ? 2048 : 640)) {
     a.shape.pairs = 1;
     // a large histogram has a copy in each block's shared memory: fewer, larger blocks

@@ -244,3 +244,36 @@ def test_plasma_pulse_gives_the_same_bits_in_every_shape(env, pol):
     for launch in (dict(block=64, grid_cache=1), dict(block=64, pairs=1), dict(block=64, pairs=1, grid_cache=1),
                    dict(block=64, pairs=1, grid_cache=2)):
         _same(base, gpu_push(*args, grid=cells, launch=launch)[0])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("per_set", [60, 257])
+def test_default_shape_batched_with_a_grid(per_set):
+    """Many small sets on a per-cell grid: the default pads a set to tiles of 64
+    (a tile counter's final value shows the tiles: their number and one more pop
+    for each block), and the states are those of an explicit shape."""
+    import torch
+    from paper_2307_04843_gb300 import _lib
+    n_sets = 4096
+    n = n_sets * per_set
+    pulses = [dict(BASE, pol=p, **KINDS["gauss"]) for p in ("x", "cm")] * (n_sets // 2)
+    parts = _parts(n)
+    box = ((-4 * L, 4 * L),) * 2 + ((-5 * L, 5 * L),)
+    f = torch.as_tensor(workloads.grid_field(box, 20, amplitude=0.2)).cuda()
+    g = _lib.pack_grid((f, tuple(b[0] for b in box), tuple(b[1] for b in box)), layout="cells")
+    off = torch.arange(n_sets + 1, dtype=torch.int64, device="cuda") * per_set
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    res = []
+    for launch in (None, dict(block=128)):
+        with _lib.Handle(pulses) as h:
+            if launch:
+                h.set_launch(**launch)
+            dev = _lib.to_device(parts, "fp32")
+            ws = torch.zeros(64, dtype=torch.int32, device="cuda")
+            _lib.ap_gather_push_batched(h.h, dev, off, g, -3.0, 0.02, 4, "fp32", None, ws)
+            assert h.status() == 0
+            res.append(_lib.to_host(dev))
+        if launch is None:
+            pops = int(ws[0]) - n_sets * (-(-per_set // 64))
+            assert 0 < pops <= 64 * sms, int(ws[0])
+    _same(*res)
