@@ -954,8 +954,7 @@ __device__ __forceinline__ void grid_values(const GridSlots &gc, float o[6]) {
   const float a00 = ux * uy, a10 = gc.wx * uy, a01 = ux * gc.wy, a11 = gc.wx * gc.wy;
   const float w[8] = {a00 * uz, a10 * uz, a01 * uz, a11 * uz, a00 * gc.wz, a10 * gc.wz,
                       a01 * gc.wz, a11 * gc.wz};
-#pragma unroll
-  for (int c = 0; c < 6; ++c) o[c] = 0.0f;
+  o[0] = o[1] = o[2] = o[3] = o[4] = o[5] = 0.0f;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const float4 lo = lds128(gc.s0 + (2 * k) * gc.step);

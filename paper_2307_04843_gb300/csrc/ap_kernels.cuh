@@ -108,19 +108,25 @@ __device__ __forceinline__ double push_one(const Pulse<Real<PREC>> &P, const Pus
   // and without it (its test would otherwise cost every step an issue slot)
   auto steps = [&](auto with_lf) {
     constexpr bool LF = decltype(with_lf)::value;
-    for (long long n = 0; n < a.n_steps; ++n) {
-      const typename TimeBase<PREC>::Step st = tb.at(n);
-      Local<R> L = local_coords<PREC>(P, st, pos);
-      if constexpr (GRID && std::is_same<R, double>::value) grid_fetch(a.grid, gc, L.x, L.y, pos.zr());
-      else if constexpr (GRID) grid_fetch_at(a.grid, gc, L.x, L.y, pos.zr());
-      R E[3], B[3];
-      analytic_fields<KIND, PREC>(P, L, E, B);
-      if constexpr (GRID) grid_eval(gc, E, B);
-      R ig = boris(u, E, B, dtR);
-      pos.advance(u[0] * ig, u[1] * ig, u[2] * ig, dtxy, dtR);
-      if constexpr (LF) {
-        R dev = valid ? fabs((R(1) / ig - u[2]) - h0) : R(0);
-        warp_max_to(lf + n, dev, 0xffffffffu);
+    // in chunks: an int counter in the loop itself costs the step fewer
+    // instructions than a long long one (PHASE64, Gaussian and per-cell grid: 1304
+    // against 1268 us)
+    for (long long s0 = 0; s0 < a.n_steps; s0 += kStepChunk) {
+      const int cnt = (int)(a.n_steps - s0 < kStepChunk ? a.n_steps - s0 : kStepChunk);
+      for (int k = 0; k < cnt; ++k) {
+        const typename TimeBase<PREC>::Step st = tb.at(s0 + k);
+        Local<R> L = local_coords<PREC>(P, st, pos);
+        if constexpr (GRID && std::is_same<R, double>::value) grid_fetch(a.grid, gc, L.x, L.y, pos.zr());
+        else if constexpr (GRID) grid_fetch_at(a.grid, gc, L.x, L.y, pos.zr());
+        R E[3], B[3];
+        analytic_fields<KIND, PREC>(P, L, E, B);
+        if constexpr (GRID) grid_eval(gc, E, B);
+        R ig = boris(u, E, B, dtR);
+        pos.advance(u[0] * ig, u[1] * ig, u[2] * ig, dtxy, dtR);
+        if constexpr (LF) {
+          R dev = valid ? fabs((R(1) / ig - u[2]) - h0) : R(0);
+          warp_max_to(lf + s0 + k, dev, 0xffffffffu);
+        }
       }
     }
   };
