@@ -1442,6 +1442,7 @@ __device__ __forceinline__ void row_put(T *__restrict__ row, int n, W v, bool ac
     if constexpr (sizeof(T) == 4) x = make_float4(vt, vt, vt, vt);
     else x = make_double2(vt, vt);
     if (lane < head) row[lane] = vt;
+#pragma unroll 4
     for (int i = lane; i < nv; i += 32) rv[i] = x;
     for (int i = tail + lane; i < n; i += 32) row[i] = vt;
   }
@@ -1449,12 +1450,13 @@ __device__ __forceinline__ void row_put(T *__restrict__ row, int n, W v, bool ac
 
 // Plane waves (Eqs. plane_func, plane_b) depend on z and t only.  A row of
 // nx nodes (fixed y, z) holds two z positions: the whole node z_k (Ex, Ey,
-// Bz) and the half node z_k + dz/2 (Ez, Bx, By).  Each warp takes a contiguous
-// run of rows and evaluates the field once per z index at each position it
-// needs (every lane computes the same value), then streams each requested
-// component along its rows with 16-byte stores, so for nx >= 32 the kernel is
-// bound by the stores, not the arithmetic.
-template <int PREC, typename T>
+// Bz) and the half node z_k + dz/2 (Ez, Bx, By).  A warp evaluates the field
+// (every lane computes the same value) and streams each requested component
+// along its rows with 16-byte stores, so for nx >= 32 the kernel is bound by the
+// stores, not the arithmetic.
+// RUNS: each warp takes a contiguous run of rows and evaluates once per z index; otherwise rows are dealt out in turn, one
+// evaluation per row.  plane_runs says which, with the times of both.
+template <int PREC, typename T, bool RUNS>
 __global__ void __launch_bounds__(256) nodes_plane_kernel(const __grid_constant__ Pulse<Real<PREC>> P,
                                                           const __grid_constant__ NodeArgs a) {
   using R = Real<PREC>;
@@ -1468,50 +1470,76 @@ __global__ void __launch_bounds__(256) nodes_plane_kernel(const __grid_constant_
   const long long rows = (long long)a.ny * a.nz;
   const int lane = threadIdx.x & 31;
   const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+  const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   TimeBase<PREC> tb;
   tb.init(P, a.t, 0.0);
   const typename TimeBase<PREC>::Step st = tb.at(0);
-  const long long per = (rows + warps - 1) / warps;
-  const long long r0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per;
-  const long long r1 = r0 + per < rows ? r0 + per : rows;
-  int kcur = -1;
-  R v[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
-  for (long long r = r0; r < r1; ++r) {
-    const int k = (int)(r / a.ny);
-    if (k != kcur) {
-      kcur = k;
+  auto eval = [&](int k, R v[6]) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (!need[h]) continue;
-        const float oz = h ? 0.5f : 0.0f;
-        Pos<PREC> pos;
-        if constexpr (PREC == AP_FP32_PHASEFF) {
-          pos.x = FF{0.0f, 0.0f};
-          pos.y = FF{0.0f, 0.0f};
-          pos.z = node_coord_ff((float)k + oz, a.lo_hi[2], a.lo_lo[2], a.d_hi[2], a.d_lo[2]);
-        } else {
-          pos.load(0.0, 0.0, fma((double)k + oz, a.d[2], a.lo[2]));
-        }
-        Local<R> L = local_coords<PREC>(P, st, pos);
-        R E[3], B[3];
-        node_values<AP_PLANE, PREC>(P, L, a.current, E, B);
-        if (h == 0) {
-          v[0] = E[0];
-          v[1] = E[1];
-          v[5] = B[2];
-        } else {
-          v[2] = E[2];
-          v[3] = B[0];
-          v[4] = B[1];
-        }
+    for (int h = 0; h < 2; ++h) {
+      if (!need[h]) continue;
+      const float oz = h ? 0.5f : 0.0f;
+      Pos<PREC> pos;
+      if constexpr (PREC == AP_FP32_PHASEFF) {
+        pos.x = FF{0.0f, 0.0f};
+        pos.y = FF{0.0f, 0.0f};
+        pos.z = node_coord_ff((float)k + oz, a.lo_hi[2], a.lo_lo[2], a.d_hi[2], a.d_lo[2]);
+      } else {
+        pos.load(0.0, 0.0, fma((double)k + oz, a.d[2], a.lo[2]));
+      }
+      Local<R> L = local_coords<PREC>(P, st, pos);
+      R E[3], B[3];
+      node_values<AP_PLANE, PREC>(P, L, a.current, E, B);
+      if (h == 0) {
+        v[0] = E[0];
+        v[1] = E[1];
+        v[5] = B[2];
+      } else {
+        v[2] = E[2];
+        v[3] = B[0];
+        v[4] = B[1];
       }
     }
+  };
+  auto put = [&](long long r, const R v[6]) {
     for (int i = 0; i < a.n_comp; ++i) {
       const int c = a.comp[i];
       const R val = c == 0 ? v[0] : c == 1 ? v[1] : c == 2 ? v[2] : c == 3 ? v[3] : c == 4 ? v[4] : v[5];
       row_put<T, W>(static_cast<T *>(a.f[c]) + r * a.nx, a.nx, (W)val, a.accumulate != 0, lane);
     }
+  };
+  if constexpr (RUNS) {
+    const long long per = (rows + warps - 1) / warps;
+    const long long r0 = wid * per, r1 = r0 + per < rows ? r0 + per : rows;
+    int kcur = -1;
+    R v[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
+    for (long long r = r0; r < r1; ++r) {
+      const int k = (int)(r / a.ny);
+      if (k != kcur) eval(k, v);
+      kcur = k;
+      put(r, v);
+    }
+  } else {
+    for (long long r = wid; r < rows; r += warps) {
+      R v[6] = {R(0), R(0), R(0), R(0), R(0), R(0)};
+      eval((int)(r / a.ny), v);
+      put(r, v);
+    }
   }
+}
+
+// Whether plane-wave rows go in runs (see nodes_plane_kernel).  Runs save
+// evaluations, which counts where one is in double or the rows are short; dealt
+// out in turn, neighbouring rows are written at the same time, which counts for
+// wide rows, above all where they end inside a 128-byte line.  Measured, rows in
+// turn / in runs, all components, us: float nodes 250 x 133 x 251 48.8 / 53.4,
+// 1000 x 140 x 140 83.5 / 91.3, 400 x 200 x 200 accumulated 75.6 / 82.4, but
+// 64 x 512 x 300 139 / 96; double nodes 256^3 136 / 130, accumulated 159 /
+// 139, 1000 x 140 x 140 156 / 166, accumulated 160 / 146; evaluated in double
+// 256^3 475 / 138.
+inline bool plane_runs(int precision, const NodeArgs &a) {
+  if (precision != AP_FP32_PHASEFF || a.nx < 192) return true;
+  return a.f64 && (a.accumulate || (a.nx * sizeof(double)) % 128 == 0);
 }
 
 template <int KIND, int PREC>
@@ -1527,8 +1555,10 @@ int launch_nodes_t(const Pulse<Real<PREC>> &P, const NodeArgs &a, void *stream) 
       if (gx < 1) gx = 1;
       const dim3 grid((unsigned)gx, 1u);
       cudaStream_t s = static_cast<cudaStream_t>(stream);
-      if (a.f64) nodes_plane_kernel<PREC, double><<<grid, block, 0, s>>>(P, a);
-      else nodes_plane_kernel<PREC, float><<<grid, block, 0, s>>>(P, a);
+      const bool runs = plane_runs(PREC, a);
+      auto kern = a.f64 ? (runs ? nodes_plane_kernel<PREC, double, true> : nodes_plane_kernel<PREC, double, false>)
+                        : (runs ? nodes_plane_kernel<PREC, float, true> : nodes_plane_kernel<PREC, float, false>);
+      kern<<<grid, block, 0, s>>>(P, a);
       return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
     }
   }
