@@ -1176,19 +1176,20 @@ __global__ void __launch_bounds__(256) nodes_row_kernel(const __grid_constant__ 
   }
 }
 
-// The row kernel with two nodes per lane and iteration (float-float, LG beams
-// and the flying-focus sum):
+// The row kernel with two nodes per lane and iteration (float-float, beams):
 // lane l takes x = l + 64 m and l + 64 m + 32, the two halves of every packed
 // value (ap_pair.cuh), so the position part of the six evaluations -- the
 // only per-node work -- issues once for both nodes.  Each warp takes a
 // contiguous run of rows, so the z/t part of its rows (carrier phase and
-// envelope argument) is computed only when the z index changes, once per run
-// of up to ny rows, instead of once per row.  Stores stay coalesced: the warp writes 32 consecutive
-// elements for each half.
+// envelope argument; for Gaussian beams also the envelope and q) is computed
+// only when the z index changes, once per run of up to ny rows, instead of once
+// per row.  Stores stay coalesced: the warp writes 32 consecutive elements for
+// each half.
 template <int KIND, typename T>
 __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_constant__ Pulse<float> P,
                                                              const __grid_constant__ NodeArgs a) {
   using W = typename std::conditional<(sizeof(T) > sizeof(float)), T, float>::type;
+  constexpr bool kGaussZ = KIND == AP_GAUSS || KIND == AP_FLYING_CF;
   unsigned want = 0u;
   for (int q = 0; q < a.n_comp; ++q) want |= 1u << a.comp[q];
   const long long rows = (long long)a.ny * a.nz;
@@ -1204,6 +1205,7 @@ __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_consta
   constexpr int kOx[6] = {1, 0, 0, 0, 1, 1}, kOy[6] = {0, 1, 0, 1, 0, 1}, kOz[6] = {0, 0, 1, 1, 1, 0};
   int kcur = -1;
   Local<F2> Lz[2];
+  BeamZ<F2> Bz[2];
   // (j, k) of the run's first row by one division, then stepped row by row
   int k = (int)(r0 / a.ny);
   int j = (int)(r0 - (long long)k * a.ny);
@@ -1221,7 +1223,12 @@ __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_consta
         pos.y = FF{0.0f, 0.0f};
         pos.z = node_coord_ff((float)k + (h ? 0.5f : 0.0f), a.lo_hi[2], a.lo_lo[2], a.d_hi[2], a.d_lo[2]);
         const Local<float> l = local_coords<AP_FP32_PHASEFF>(P, st, pos);
-        Lz[h] = Local<F2>{F2(l.x), F2(l.y), F2(l.dz), F2(l.psi), F2(l.eta), F2(l.T), F2(l.phi_hi), F2(l.phi_lo)};
+        if constexpr (kGaussZ) {
+          const BeamZ<float> b = gauss_z<KIND == AP_FLYING_CF>(P, l);
+          Bz[h] = BeamZ<F2>{Cx<F2>{F2(b.q.re), F2(b.q.im)}, F2(b.amp_mul), F2(b.l2), F2(b.psi)};
+        } else {
+          Lz[h] = Local<F2>{F2(l.x), F2(l.y), F2(l.dz), F2(l.psi), F2(l.eta), F2(l.T), F2(l.phi_hi), F2(l.phi_lo)};
+        }
       }
     }
     const float ys[2] = {fmaf((float)j, a.d_hi[1], a.lo_hi[1]), fmaf((float)j + 0.5f, a.d_hi[1], a.lo_hi[1])};
@@ -1239,10 +1246,14 @@ __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_consta
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
         F2 E[3], B[3];
-        Local<F2> L = Lz[kOz[c]];
-        L.x = xs[kOx[c]];
-        L.y = F2(ys[kOy[c]]);
-        analytic_fields<KIND, AP_FP32_PHASEFF, F2>(P, L, E, B);
+        if constexpr (kGaussZ) {
+          gauss_xy(P, Bz[kOz[c]], xs[kOx[c]], F2(ys[kOy[c]]), E, B);
+        } else {
+          Local<F2> L = Lz[kOz[c]];
+          L.x = xs[kOx[c]];
+          L.y = F2(ys[kOy[c]]);
+          analytic_fields<KIND, AP_FP32_PHASEFF, F2>(P, L, E, B);
+        }
         v[c] = c < 3 ? E[c] : B[c - 3];
       }
 #pragma unroll
@@ -1271,8 +1282,9 @@ __global__ void __launch_bounds__(256) nodes_row_pair_kernel(const __grid_consta
 // store bandwidth; this is bound by the stores (256^3, 402 MB: 88.5 -> 72.6 us, 5.5 TB/s).  The
 // factors are made with the accurate library functions (each is used by tens of nodes), so that their
 // product is as good as one approximate exponential was.
-// VEC: four consecutive columns per lane and 16-byte accesses (rows aligned to
-// 16 bytes); otherwise columns 32 apart.
+// VEC: four consecutive columns per lane and 16-byte accesses (float rows aligned
+// to 16 bytes); otherwise columns 32 apart, stores only.  slab_wins says which
+// shapes come here.
 constexpr int kSlabCols = 128;
 constexpr int kSlabRows = 32;  // at most; one lane makes one row's coefficients
 
@@ -1288,7 +1300,6 @@ __device__ __forceinline__ Cx<float> beam_factor(float a, Cx<float> q, float tur
 template <int KIND, typename T, bool VEC>
 __global__ void __launch_bounds__(256) nodes_slab_kernel(const __grid_constant__ PulseHead<float> P,
                                                          const __grid_constant__ NodeArgs a) {
-  using W = typename std::conditional<(sizeof(T) > sizeof(float)), T, float>::type;
   __shared__ float4 s_row[8][kSlabRows][4];
   unsigned want = 0u;
   for (int q = 0; q < a.n_comp; ++q) want |= 1u << a.comp[q];
@@ -1401,7 +1412,7 @@ __global__ void __launch_bounds__(256) nodes_slab_kernel(const __grid_constant__
         } else {
 #pragma unroll
           for (int m = 0; m < 4; ++m)
-            if (i0 + 32 * m < a.nx) f[32 * m] = a.accumulate ? (T)((W)f[32 * m] + (W)v[c][m]) : (T)v[c][m];
+            if (i0 + 32 * m < a.nx) f[32 * m] = (T)v[c][m];
         }
       }
     }
@@ -1446,6 +1457,32 @@ __device__ __forceinline__ void row_put(T *__restrict__ row, int n, W v, bool ac
     for (int i = lane; i < nv; i += 32) rv[i] = x;
     for (int i = tail + lane; i < n; i += 32) row[i] = vt;
   }
+}
+
+// Whether a Gaussian beam's nodes go in slabs (nodes_slab_kernel) or row by row
+// (nodes_row_pair_kernel, two columns of 32 per pass).  A slab pays its set-up, 16
+// exponentials and sines per lane, for each z index and 128 columns, and does the
+// work of 128 columns also where fewer are left; without 16-byte accesses
+// (double nodes, unaligned rows) it stores and sums by single elements, where
+// the row kernel is as wide; and where rows end inside a 32-byte sector, the
+// sectors at the slabs' edges are written in two parts far apart in time.
+// Measured, slabs / rows, us (1.7e7 nodes where ny allows):
+//   float nodes, stored: nx 256 78 / 93, with ny = 1, 2, 3 97 / 59, 107 / 97, 84 / 96;
+//     nx 64 with ny = 3, 5, 8 67 / 53, 65 / 61, 55 / 61; nx 160 with ny = 3, 4 69 / 65, 61 /
+//     63; unaligned, nx 33 with ny = 6, 12 99 / 84, 100 / 100; rows that end inside a
+//     sector: nx 300 129 / 100, nx 180 138 / 100, nx 250 123 / 108, with ny = 3 99 / 110;
+//   float nodes, summed: nx 256 229 / 397, nx 64 360 / 388, with ny = 1 61 / 44, nx 32
+//     656 / 427; unaligned, nx 250 679 / 400;
+//   double nodes, stored: nx 64 188 / 102, nx 160 156 / 122, nx 250 207 / 191, nx 256
+//     180 / 182, nx 1000 182 / 201; summed: nx 256 717 / 534.
+inline bool slab_wins(const NodeArgs &a, bool vec) {
+  const int slabs = (a.nx + kSlabCols - 1) / kSlabCols, pairs = (a.nx + 63) / 64;
+  const bool full = pairs == 2 * slabs;
+  if (a.f64) return !a.accumulate && full && a.nx % 4 == 0 && a.ny >= 4;
+  if (a.accumulate) return vec && (pairs > slabs || (a.nx == 64 && a.ny > 2));
+  if (slabs > 1 && a.nx % 8 != 0) return full && a.ny >= 3 && a.ny < 6;
+  if (!vec && pairs == slabs) return a.ny >= 12;
+  return (long long)a.ny * pairs >= 6LL * slabs;
 }
 
 // Plane waves (Eqs. plane_func, plane_b) depend on z and t only.  A row of
@@ -1573,18 +1610,18 @@ int launch_nodes_t(const Pulse<Real<PREC>> &P, const NodeArgs &a, void *stream) 
       if constexpr (KIND == AP_GAUSS || KIND == AP_FLYING_CF) {
         bool vec = !a.f64 && a.nx % 4 == 0;
         for (int i = 0; i < a.n_comp; ++i) vec = vec && (reinterpret_cast<uintptr_t>(a.f[a.comp[i]]) & 15u) == 0;
-        auto kern = a.f64 ? nodes_slab_kernel<KIND, double, false>
-                    : vec ? nodes_slab_kernel<KIND, float, true> : nodes_slab_kernel<KIND, float, false>;
-        // one resident wave, and at least four rows for each warp's set-up
-        const long long units = (long long)((a.nx + kSlabCols - 1) / kSlabCols) * rows;
-        long long gp = (long long)a.sm_count * occupancy_blocks(kern, block, 0);
-        if (gp > (units + 31) / 32) gp = (units + 31) / 32;
-        kern<<<(unsigned)gp, block, 0, s>>>(P, a);
-        return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
+        if (slab_wins(a, vec)) {
+          auto kern = a.f64 ? nodes_slab_kernel<KIND, double, false>
+                      : vec ? nodes_slab_kernel<KIND, float, true> : nodes_slab_kernel<KIND, float, false>;
+          // one resident wave, and at least four rows for each warp's set-up
+          const long long units = (long long)((a.nx + kSlabCols - 1) / kSlabCols) * rows;
+          long long gp = (long long)a.sm_count * occupancy_blocks(kern, block, 0);
+          if (gp > (units + 31) / 32) gp = (units + 31) / 32;
+          kern<<<(unsigned)gp, block, 0, s>>>(P, a);
+          return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
+        }
       }
-      // the other beams: two nodes per lane, packed; one resident wave of
-      // blocks, each warp a contiguous run of rows
-      else {
+      {  // two nodes per lane, packed; one resident wave of blocks, each warp a contiguous run of rows
         auto kern = a.f64 ? nodes_row_pair_kernel<KIND, double> : nodes_row_pair_kernel<KIND, float>;
         long long gp = (long long)a.sm_count * occupancy_blocks(kern, block, 0);
         if (gp > (rows + 7) / 8) gp = (rows + 7) / 8;
