@@ -999,6 +999,15 @@ int launch_push_ff_t(const Pulse<float> &P, const PushArgs &a, void *stream) {
   const size_t head = push_smem_head<AP_FP32_PHASEFF, GRID, NP>(block);
   const size_t smem = head + (a.diag.hist ? (size_t)a.diag.bins * sizeof(uint32_t) : 0);
   if (set_smem(kern, smem) != AP_OK) return AP_ERR_CUDA;
+  // Node corners: four blocks of 128 per SM and the rest of the 256 KB to the L1
+  // cache.  At 80 registers six fit, whose slots would leave it 30 KB, and the
+  // gather from plain component arrays (48 loads of 4 bytes per cell, sectors
+  // shared by neighbouring corners) lives from it (256^3 grid, 2e6 particles, 50
+  // steps: plain arrays 2519 us with the driver's choice, 1305 so; packed nodes
+  // 965 / 870).
+  if (GRID == kGridNodes &&
+      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 60) != cudaSuccess)
+    return AP_ERR_CUDA;
   const long long per_block = (long long)NP * block;
   const long long want = (a.n + per_block - 1) / per_block;
   int per_sm = a.shape.blocks_per_sm > 0 ? a.shape.blocks_per_sm : occupancy_blocks(kern, block, smem);
