@@ -255,8 +255,9 @@ typedef struct {
                                          three per-node phase constants in shared memory) */
 
 /* Launch shape, chosen by the autotuner (block 0 = library default).  While
- * none is set, the library picks block, pairs and grid_cache by the call's
- * size, arithmetic and grid layout. */
+ * none is set (no ap_set_launch yet, or the last one with NULL or with every
+ * field 0), the library picks block, pairs and grid_cache by the call's size,
+ * arithmetic and grid layout. */
 typedef struct {
   int32_t block;          /* threads per block, multiple of 32, <= 1024 */
   int32_t blocks_per_sm;  /* persistent kernels: resident blocks per SM */

@@ -757,7 +757,8 @@ int ap_set_launch(ap_handle h, const ap_launch_cfg *cfg) {
   if (cfg->pairs != 0 && cfg->pairs != 1) return AP_ERR_ARG;
   if (cfg->tile < 0 || cfg->tile > (1 << 24)) return AP_ERR_ARG;
   h->shape = apt::LaunchShape{cfg->block, cfg->blocks_per_sm, cfg->grid_cache, cfg->pairs, cfg->tile};
-  h->shape_set = true;
+  // all zero asks for nothing: the library's own choice, as with no cfg
+  h->shape_set = cfg->block || cfg->blocks_per_sm || cfg->grid_cache || cfg->pairs || cfg->tile;
   return AP_OK;
 }
 

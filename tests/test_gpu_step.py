@@ -277,3 +277,26 @@ def test_default_shape_batched_with_a_grid(per_set):
             pops = int(ws[0]) - n_sets * (-(-per_set // 64))
             assert 0 < pops <= 64 * sms, int(ws[0])
     _same(*res)
+
+
+@pytest.mark.gpu
+def test_set_launch_without_a_shape_gives_the_default_back():
+    """Handle.set_launch() after an explicit shape: the tiles of the next batched
+    call (see the tile counter) are those of a fresh handle."""
+    import torch
+    from paper_2307_04843_gb300 import _lib
+    n_sets, per_set = 4096, 257
+    parts = _parts(n_sets * per_set)
+    box = ((-4 * L, 4 * L),) * 2 + ((-5 * L, 5 * L),)
+    f = torch.as_tensor(workloads.grid_field(box, 20, amplitude=0.2)).cuda()
+    g = _lib.pack_grid((f, tuple(b[0] for b in box), tuple(b[1] for b in box)), layout="cells")
+    off = torch.arange(n_sets + 1, dtype=torch.int64, device="cuda") * per_set
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    with _lib.Handle([dict(BASE, pol="x", **KINDS["gauss"])] * n_sets) as h:
+        for launch, tile in ((dict(block=256), 256), (dict(), 64)):
+            h.set_launch(**launch)
+            dev = _lib.to_device(parts, "fp32")
+            ws = torch.zeros(64, dtype=torch.int32, device="cuda")
+            _lib.ap_gather_push_batched(h.h, dev, off, g, -3.0, 0.02, 1, "fp32", None, ws)
+            assert h.status() == 0
+            assert 0 < int(ws[0]) - n_sets * (-(-per_set // tile)) <= 64 * sms
