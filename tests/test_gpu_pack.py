@@ -58,3 +58,38 @@ def test_cell_coefficients_of_huge_and_nonfinite_corners():
     # the double differences drop a corner of 1 beside one of 3e38; the tolerance above covers that
     err = np.abs(out[fin].astype(np.float64) - ref[fin])
     assert np.all(err <= 2.0 ** -24 * np.abs(ref[fin]) + 2.0 ** -45 * 3.0e38)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(2, 2, 2), (3, 5, 33), (20, 33, 34)])
+@pytest.mark.parametrize("form", ["wide", "near", "linear"])
+def test_cell_coefficients_of_cancelling_corners(shape, form):
+    """Differences that cancel to their last bits, each cell against exact
+    rational differences, on its own scale: half a unit in the last place, a
+    fiftieth of that, and 2^-60 of the cell's largest corner.  Wide: corners of 1 beside ones of 1e-8, so that first
+    differences have low parts of 24 bits; near: corners that agree to 1e-4;
+    linear: fields whose second differences are rounding alone."""
+    from fractions import Fraction
+    rng = np.random.default_rng(sum(shape))
+    if form == "wide":
+        f = np.where(np.arange(shape[2]) % 2 == 0, 1.0, 1e-8 * (1.0 + rng.random((6,) + shape)))
+    elif form == "near":
+        f = 1.0 + 1e-4 * rng.standard_normal((6,) + shape)
+    else:
+        z, y, x = np.meshgrid(*(np.arange(n) for n in shape), indexing="ij")
+        f = np.stack([1.0 + 0.1 * (c + 1) * x - 0.37 * y + 1e-3 * z for c in range(6)])
+    f = f.astype(np.float32)
+    out = _packed(f)
+    nz, ny, nx = (v - 1 for v in shape)
+    for _ in range(400):
+        c, k, j, i = (int(rng.integers(0, n)) for n in (6, nz, ny, nx))
+        v = {(x, y, z): Fraction(float(f[c, k + z, j + y, i + x])) for x in (0, 1) for y in (0, 1) for z in (0, 1)}
+        a = [v[0, 0, 0], v[1, 0, 0] - v[0, 0, 0], v[0, 1, 0] - v[0, 0, 0], v[0, 0, 1] - v[0, 0, 0]]
+        a.append(v[1, 1, 0] - v[1, 0, 0] - a[2])
+        a.append(v[0, 1, 1] - v[0, 1, 0] - a[3])
+        a.append(v[1, 0, 1] - v[1, 0, 0] - a[3])
+        a.append(v[1, 1, 1] - v[1, 1, 0] - v[1, 0, 1] + v[1, 0, 0] - a[5])
+        big = max(abs(x) for x in v.values())
+        for p, want in enumerate(a):
+            got = Fraction(float(out[c, k, j, i, p]))
+            assert abs(got - want) <= abs(want) * Fraction(51, 50) / 2 ** 24 + big / 2 ** 60, (c, k, j, i, p)
