@@ -148,13 +148,18 @@ struct SplitArgs {
 // window.  The envelope is 2^-(u^{2g}) of the scaled argument u.
 constexpr int kOrderAny = 0, kSin2 = -1;
 
-// s^n, n >= 1; N > 0: n = N, by squaring
+// s^n by squaring; N = 0: 0 <= n <= 15 at run time (the bits of n are the same
+// for all threads), N > 0: n = N
 template <int N>
 __device__ __forceinline__ F2 upow(F2 s, int n) {
   if constexpr (N == 0) {
-    F2 p = s;
-    for (int i = 1; i < n; ++i) p = rmul(p, s);
-    return p;
+    F2 q = n & 1 ? s : F2(1.0f);
+    s = rmul(s, s);
+    if (n & 2) q = rmul(q, s);
+    s = rmul(s, s);
+    if (n & 4) q = rmul(q, s);
+    if (n & 8) q = rmul(q, rmul(s, s));
+    return q;
   } else if constexpr (N == 1) {
     return s;
   } else if constexpr (N % 2 == 0) {
@@ -250,7 +255,8 @@ __global__ void __launch_bounds__(MAXT) split_line_kernel(const __grid_constant_
         m0 = window2(u0, sa.env_w);
         m1 = window2(u1, sa.env_w);
       } else {
-        m0 = exp2_neg(upow<G>(rmul(u0, u0), sa.g));
+        const F2 s0 = rmul(u0, u0);
+        m0 = exp2_neg(G == kOrderAny ? rmul(upow<0>(s0, sa.g - 1), s0) : upow<G>(s0, 0));
         if constexpr (G == 1) {
           m1 = exp2_neg(rmul(u1, u1));
           th = rmul(F2(sa.k1), u1);
@@ -260,8 +266,7 @@ __global__ void __launch_bounds__(MAXT) split_line_kernel(const __grid_constant_
           // held where the envelope is zero, as th and A would overflow (see
           // sg_bound; the compiled orders are for lines on which they do not)
           if constexpr (G == kOrderAny) s = F2(fminf(s.x, sa.s_max), fminf(s.y, sa.s_max));
-          F2 q = F2(1.0f);
-          if (G > 1 || sa.g > 1) q = upow<(G > 1 ? G - 1 : 0)>(s, sa.g - 1);
+          const F2 q = upow<(G > 1 ? G - 1 : 0)>(s, sa.g - 1);
           m1 = exp2_neg(rmul(q, s));
           th = rmul(F2(sa.k1), rmul(u1, q));
           A = rfma(F2(sa.k2), q, rfma(rmul(F2(-0.5f), th), th, F2(1.0f)));
@@ -300,7 +305,13 @@ template <int C, int MAXT>
 int launch_split(const SplitArgs &sa, void *stream) {
   if (sa.env == AP_ENV_SIN2) return launch_split_g<C, MAXT, kSin2>(sa, stream);
   if (sa.g == 1) return launch_split_g<C, MAXT, 1>(sa, stream);
-  if (sa.g == 4 && sa.finite) return launch_split_g<C, MAXT, 4>(sa, stream);
+  // low orders (2 to 4) have their powers compiled in; above, and where the
+  // powers need holding, the order is a run-time number (304 lines of 4096 nodes,
+  // 500 steps: orders 2, 3, 4 777, 816, 820 us, 5 and 8 1014, 1027 us; with a loop
+  // over the order 930, 1037, -, 1139, 1305)
+  if (sa.finite && sa.g == 2) return launch_split_g<C, MAXT, 2>(sa, stream);
+  if (sa.finite && sa.g == 3) return launch_split_g<C, MAXT, 3>(sa, stream);
+  if (sa.finite && sa.g == 4) return launch_split_g<C, MAXT, 4>(sa, stream);
   return launch_split_g<C, MAXT, kOrderAny>(sa, stream);
 }
 
