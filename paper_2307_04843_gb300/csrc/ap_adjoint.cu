@@ -761,7 +761,8 @@ __device__ __forceinline__ void reverse_step_pair(const PT &P, const StepBase &s
   using R = F2;
   const FastPulse &F = P.fast;
   // unit fields, as in unit_fields_beam
-  const R eta = rfma(zhi, R(F.c_eta), R(st.y));
+  R eta = rfma(zhi, R(F.c_eta), R(st.y));
+  if constexpr (ENV != kEnvGauss) eta = rfma(zhi, R(F.c_eta_lo), eta);
   R mul, g;
   envelope_fast<ENV>(P, eta, mul, g);
   const R zn = KIND == AP_FLYING_CF ? rfma(zhi, R(F.c_zn), R(st.z)) : rmul(zhi, R(F.c_zn));

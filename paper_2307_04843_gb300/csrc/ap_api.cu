@@ -372,13 +372,20 @@ void derive(const ap_pulse_desc &d, Pulse<double> &P, Pulse<float> &F) {
                       : P.env == AP_ENV_SIN2 || P.env == AP_ENV_SGAUSS ? P.env_a : 1.0;
   S.env_len = (float)(1.0 / senv);
   S.env_w = (float)(P.env_a * P.env_b);
-  // The factor of Z is rounded to float; the factor of T is what belongs to the
-  // rounded one, in two floats.  Two factors rounded each for itself would leave
-  // 2^-24 (t - t_f) of eta where the two terms cancel; this one scales eta as a
-  // whole by 1 + 2^-25 at most.
-  S.c_eta = (float)(-senv * P.inv_vg * S.z_len);
-  const double sT = -(double)S.c_eta / (P.inv_vg * S.z_len);
-  split(std::isfinite(sT) ? sT : senv, S.s_env, S.s_env_lo);
+  // Factors rounded to one float each would leave 2^-24 (t - t_f) of eta where the
+  // two terms cancel.  For zeta and for a Gaussian envelope it is enough that they
+  // belong together, the factor of T in two floats made from the rounded factor of
+  // Z: that scales the argument as a whole, by 1 + 2^-25 at most.  The other
+  // envelopes have edges and high powers, and take both factors in two floats (one
+  // operation more; 3 % of the batched Gaussian push, where it is not needed).
+  split(-senv * P.inv_vg * S.z_len, S.c_eta, S.c_eta_lo);
+  double sT = senv;
+  if (P.env == AP_ENV_GAUSS) {
+    S.c_eta_lo = 0.0f;
+    const double s = -(double)S.c_eta / (P.inv_vg * S.z_len);
+    if (std::isfinite(s)) sT = s;
+  }
+  split(sT, S.s_env, S.s_env_lo);
   S.c_zn = (float)(-P.inv_zR * S.z_len);
   split(-(double)S.c_zn * P.beta_f / S.z_len, S.c_tz, S.c_tz_lo);
   S.c_a = (float)(P.inv_w0sq * log2e);

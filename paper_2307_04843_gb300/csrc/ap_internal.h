@@ -35,10 +35,9 @@ struct FastPulse {
   double turn0;           // carrier phase that the frame adds (turns)
   float s_env, s_env_lo, env_len;  // scale of the envelope argument (hi, lo), and its inverse
   float env_w;            // half-width of the sin^2 window, scaled
-  // eta s_env = s_env T + c_eta Z, -zeta = c_zn Z + c_tz T; the factors of T
-  // (hi, lo) are made from the rounded factors of Z, so that the two terms
-  // cancel exactly far from the focus
-  float c_eta, c_zn, c_tz, c_tz_lo;
+  // eta s_env = s_env T + c_eta Z and -zeta = c_zn Z + c_tz T, the factors of T (hi,
+  // lo) such that the two terms cancel far from the focus (see derive)
+  float c_eta, c_eta_lo, c_zn, c_tz, c_tz_lo;
   float c_a;              // log2(e) / w0^2
   float A, Abr, Ace, Acb;  // E_perp, B_perp, E_z, B_z per unit field
   float lg_n[6][kLgMaxP];  // the Laguerre recurrences with the subtracted terms' signs in

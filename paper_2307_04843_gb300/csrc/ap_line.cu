@@ -133,7 +133,7 @@ struct SplitArgs {
   int env, g;               // envelope kind; order of the super-Gaussian (Gaussian: 1)
   float zs_hi, zs_lo;       // k / 2 pi
   float zf_hi, zf_lo;
-  float su_vg;              // scale of the envelope argument over v_g
+  float su_vg, su_vg_lo;    // scale of the envelope argument over v_g
   float hu;                 // dt/2 in the scaled argument
   bool finite;              // th and A stay finite over all nodes and steps of the call
   float s_max;              // square of the scaled argument from which the super-Gaussian is zero
@@ -220,7 +220,8 @@ __global__ void __launch_bounds__(MAXT) split_line_kernel(const __grid_constant_
       FF tr = two_prod(sa.zs_hi, dz.hi);
       tr.lo = __fadd_rn(tr.lo, __fmaf_rn(sa.zs_hi, dz.lo, __fmul_rn(sa.zs_lo, dz.hi)));
       const float turn = __fadd_rn(__fsub_rn(tr.hi, round_magic(tr.hi)), tr.lo);
-      const float ek = __fmul_rn(sa.su_vg, __fadd_rn(dz.hi, dz.lo));
+      const float ek =
+          __fmaf_rn(sa.su_vg, dz.hi, __fmaf_rn(sa.su_vg, dz.lo, __fmul_rn(sa.su_vg_lo, dz.hi)));
       const float qk = __fmul_rn(dtf, k < nz ? (W ? W[k] : (float)a.omega_p2) : 0.0f);
       if (h) { tn.y = turn; en2.y = ek; q.y = qk; } else { tn.x = turn; en2.x = ek; q.x = qk; }
     }
@@ -340,9 +341,9 @@ SplitArgs split_args(const Pulse<double> &pd, const Pulse<float> &pf, const Line
   } else if (pd.env == AP_ENV_SIN2) {
     su = pd.env_a;
   }
-  // the scale of t - t_f from the rounded one of z - z_f (see FastPulse)
-  s.su_vg = (float)(su * pd.inv_vg);
-  split((double)s.su_vg / pd.inv_vg, s.fast.s_env, s.fast.s_env_lo);
+  // both scales in two floats: a step's and a node's terms are made once each
+  split(su, s.fast.s_env, s.fast.s_env_lo);
+  split(su * pd.inv_vg, s.su_vg, s.su_vg_lo);
   s.fast.c_tz = s.fast.c_tz_lo = 0.0f;
   GridView none;
   std::memset(&none, 0, sizeof(none));

@@ -266,7 +266,8 @@ template <int KIND, int POL, int ENV, class PT, typename R>
 __device__ __forceinline__ UnitFields<R> unit_fields_beam(const PT &P, const float4 st, R x, R y, R zhi, R zlo) {
   const FastPulse &F = P.fast;
   UnitFields<R> o;
-  const R eta = rfma(zhi, R(F.c_eta), R(st.y));
+  R eta = rfma(zhi, R(F.c_eta), R(st.y));
+  if constexpr (ENV != kEnvGauss) eta = rfma(zhi, R(F.c_eta_lo), eta);
   R mul, g;
   envelope_fast<ENV>(P, eta, mul, g);
   if constexpr (KIND == AP_PLANE) {
