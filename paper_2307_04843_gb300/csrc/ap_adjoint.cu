@@ -1119,7 +1119,9 @@ int launch_adjoint_pair(const Pulse<float> *sets, const AdjArgs &a0, void *strea
   pair_segments(aa, slots);
   aa.tape = static_cast<char *>(aa.ckpt) + sizeof(float) * PairIO::kCkpt * (size_t)aa.n_seg * (size_t)slots;
   const size_t dyn = 2 * (size_t)PairIO::kTape * kAdjBlock * sizeof(float2) + (size_t)(aa.n_sets + 1) * sizeof(long long);
-  if (allow_smem(reinterpret_cast<const void *>(kern)) != AP_OK) return AP_ERR_CUDA;
+  constexpr size_t most =
+      2 * (size_t)PairIO::kTape * kAdjBlock * sizeof(float2) + (size_t)(AP_MAX_SETS + 1) * sizeof(long long);
+  if (allow_smem(reinterpret_cast<const void *>(kern), most) != AP_OK) return AP_ERR_CUDA;
   kern<<<grid, kAdjBlock, dyn, static_cast<cudaStream_t>(stream)>>>(sets, aa);
   return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
 }
@@ -1129,7 +1131,7 @@ int launch_adjoint_t(const Pulse<Real<PREC>> *sets, const AdjArgs &aa, int grid,
   auto kern = adjoint_kernel<KIND, PREC, GRID>;
   const size_t dyn = 2 * (size_t)StateIO<PREC>::W * kAdjBlock * sizeof(typename StateIO<PREC>::T);
   // static (about 40 KB) plus dynamic shared memory passes 48 KB: opt in
-  if (allow_smem(reinterpret_cast<const void *>(kern)) != AP_OK) return AP_ERR_CUDA;
+  if (allow_smem(reinterpret_cast<const void *>(kern), dyn) != AP_OK) return AP_ERR_CUDA;
   kern<<<grid, kAdjBlock, dyn, static_cast<cudaStream_t>(stream)>>>(sets, aa);
   return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
 }

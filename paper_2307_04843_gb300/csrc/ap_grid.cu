@@ -186,7 +186,7 @@ int ap_grid_pack(const ap_grid *g, float *packed, void *stream) {
     for (int c = 0; c < 6; ++c) src.f[c] = g->f[c];
     // shared memory lets four blocks of eight warps stay resident
     const size_t smem = sizeof(float4) * 12 * kPackRow * kPackWarps;
-    if (apt::allow_smem(reinterpret_cast<const void *>(pack_cells_kernel)) != AP_OK) return AP_ERR_CUDA;
+    if (apt::allow_smem(reinterpret_cast<const void *>(pack_cells_kernel), smem) != AP_OK) return AP_ERR_CUDA;
     const long long resident = (long long)sms * 4;
     pack_cells_kernel<<<(int)(want < resident ? want : resident), 32 * kPackWarps, smem, s>>>(
         src, g->nx, g->ny, g->nz, reinterpret_cast<float4 *>(packed));

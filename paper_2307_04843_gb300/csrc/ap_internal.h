@@ -222,19 +222,13 @@ APT_DECLARE_KIND(flyingcf)
 // per-cell coefficient copy (AP_ERR_ARG when f[] is missing).
 int drop_cell_layout(GridView &v);
 
-// Lets a kernel be launched with any dynamic shared memory that fits beside its
-// static part.  The limit belongs to the kernel, not to the call: every caller
-// sets the same value, so that threads launching one kernel with different
-// sizes cannot lower it for one another between setting and launching.
-inline int allow_smem(const void *kern) {
-  int dev = 0, optin = 0;
-  cudaFuncAttributes fa;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-      cudaFuncGetAttributes(&fa, kern) != cudaSuccess)
-    return AP_ERR_CUDA;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes) ==
-                 cudaSuccess
+// Lets a kernel be launched with up to `most` bytes of dynamic shared memory, the
+// most that any call of it takes.  The limit belongs to the kernel, not to the
+// call: every caller sets the same value, so that threads launching one kernel
+// with different sizes cannot lower it for one another between setting and
+// launching.
+inline int allow_smem(const void *kern, size_t most) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) == cudaSuccess
              ? AP_OK
              : AP_ERR_CUDA;
 }

@@ -968,10 +968,16 @@ inline size_t push_smem_head(int block) {
 }
 
 // opt in above what every kernel gets without asking: 48 KB less its static
-// shared memory (up to 14 KB here: a pulse, a component table)
-template <typename K>
+// shared memory (up to 14 KB here: a pulse, a component table).  The most that a
+// push asks for: a block of 256, with a histogram of 8192 bins or the prefix of
+// AP_MAX_SETS sets.
+template <int PREC, int GRID, int NP, typename K>
 inline int set_smem(K kern, size_t smem) {
-  return smem <= 32 * 1024 ? AP_OK : allow_smem(reinterpret_cast<const void *>(kern));
+  constexpr size_t tail = (AP_MAX_SETS + 1) * sizeof(long long);
+  static_assert(tail >= 8192 * sizeof(uint32_t), "the longer tail");
+  return smem <= 32 * 1024
+             ? AP_OK
+             : allow_smem(reinterpret_cast<const void *>(kern), push_smem_head<PREC, GRID, NP>(256) + tail);
 }
 
 template <int KIND, int PREC, int GRID>
@@ -980,7 +986,7 @@ int launch_push_t(const Pulse<Real<PREC>> &P, const PushArgs &a, void *stream) {
   const int block = a.shape.block;
   const size_t head = push_smem_head<PREC, GRID>(block);
   const size_t smem = head + (a.diag.hist ? (size_t)a.diag.bins * sizeof(uint32_t) : 0);
-  if (set_smem(kern, smem) != AP_OK) return AP_ERR_CUDA;
+  if (set_smem<PREC, GRID, 1>(kern, smem) != AP_OK) return AP_ERR_CUDA;
   const long long npad = (a.n + 31) & ~31LL;
   long long want = (npad + block - 1) / block;
   int per_sm = a.shape.blocks_per_sm > 0 ? a.shape.blocks_per_sm : occupancy_blocks(kern, block, smem);
@@ -998,7 +1004,7 @@ int launch_push_ff_t(const Pulse<float> &P, const PushArgs &a, void *stream) {
   const int block = a.shape.block;
   const size_t head = push_smem_head<AP_FP32_PHASEFF, GRID, NP>(block);
   const size_t smem = head + (a.diag.hist ? (size_t)a.diag.bins * sizeof(uint32_t) : 0);
-  if (set_smem(kern, smem) != AP_OK) return AP_ERR_CUDA;
+  if (set_smem<AP_FP32_PHASEFF, GRID, NP>(kern, smem) != AP_OK) return AP_ERR_CUDA;
   // Node corners: four blocks of 128 per SM and the rest of the 256 KB to the L1
   // cache.  At 80 registers six fit, whose slots would leave it 30 KB, and the
   // gather from plain component arrays (48 loads of 4 bytes per cell, sectors
@@ -1675,7 +1681,7 @@ int launch_batch_t(const Pulse<Real<PREC>> *sets, const BatchArgs &ba, void *str
   const int block = ba.base.shape.block;
   const size_t head = push_smem_head<PREC, GRID, NP>(block);
   const size_t smem = head + (size_t)(ba.n_sets + 1) * sizeof(long long);
-  if (set_smem(kern, smem) != AP_OK) return AP_ERR_CUDA;
+  if (set_smem<PREC, GRID, NP>(kern, smem) != AP_OK) return AP_ERR_CUDA;
   int per_sm = ba.base.shape.blocks_per_sm > 0 ? ba.base.shape.blocks_per_sm
                                                 : occupancy_blocks(kern, block, smem);
   const int grid = ba.base.sm_count * per_sm;

@@ -297,7 +297,8 @@ int launch_split_g(const SplitArgs &sa, void *stream) {
   auto kern = split_line_kernel<C, MAXT, G>;
   const int block = line_block<C>(sa.line.nz);
   const size_t smem = 3 * sizeof(F2) * (size_t)C * block;
-  if (set_smem(kern, smem) != AP_OK) return AP_ERR_CUDA;
+  if (smem > 32 * 1024 && allow_smem(reinterpret_cast<const void *>(kern), 3 * sizeof(F2) * (size_t)C * MAXT) != AP_OK)
+    return AP_ERR_CUDA;
   kern<<<(unsigned)sa.line.n_lines, block, smem, static_cast<cudaStream_t>(stream)>>>(sa);
   return cudaGetLastError() == cudaSuccess ? AP_OK : AP_ERR_CUDA;
 }
@@ -372,7 +373,8 @@ template <typename T, bool APT>
 int launch_line_t(const Pulse<double> &P, const LineArgs &a, void *stream) {
   auto kern = line_kernel<T, APT>;
   const size_t smem = 4u * sizeof(T) * (size_t)a.nz;
-  if (set_smem(kern, smem) != AP_OK) return AP_ERR_CUDA;
+  constexpr size_t most = 4u * sizeof(T) * (sizeof(T) == 8 ? AP_LINE1D_MAX_NODES_F64 : AP_LINE1D_MAX_NODES_F32);
+  if (allow_smem(reinterpret_cast<const void *>(kern), most) != AP_OK) return AP_ERR_CUDA;
   int block = (a.nz + 31) / 32 * 32;
   if (block > kLineBlock) block = kLineBlock;
   kern<<<(unsigned)a.n_lines, block, smem, static_cast<cudaStream_t>(stream)>>>(P, a);

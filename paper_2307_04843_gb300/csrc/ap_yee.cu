@@ -188,7 +188,7 @@ template <typename T>
 int launch_yee1d_smem(const ap_yee1d *y, long long n_steps, void *stream) {
   const size_t smem = 2u * sizeof(T) * (size_t)y->nz;
   auto kern = yee1d_smem_kernel<T>;
-  if (allow_smem(reinterpret_cast<const void *>(kern)) != AP_OK) return AP_ERR_CUDA;
+  if (allow_smem(reinterpret_cast<const void *>(kern), 2u * sizeof(T) * AP_YEE1D_MAX_NODES) != AP_OK) return AP_ERR_CUDA;
   const double r = y->dt / y->dz;
   const double hr = 0.5 * r;
   kern<<<(unsigned)y->n_lines, kYeeBlock, smem, static_cast<cudaStream_t>(stream)>>>(
