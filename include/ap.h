@@ -249,10 +249,11 @@ typedef struct {
   double z0;
 } ap_line1d;
 
-#define AP_LINE1D_MAX_NODES_F32 12288 /* nodes per float line (the line sits in shared memory) */
-#define AP_LINE1D_MAX_NODES_F64 6144  /* nodes per double line */
-#define AP_APT1D_MAX_NODES_F32 8192   /* nodes per float line of ap_apt1d_run (it also keeps
-                                         three per-node phase constants in shared memory) */
+#define AP_LINE1D_MAX_NODES_F32 12288 /* nodes per float line (in registers up to 8192 nodes, in
+                                         shared memory above) */
+#define AP_LINE1D_MAX_NODES_F64 6144  /* nodes per double line (in shared memory) */
+#define AP_APT1D_MAX_NODES_F32 8192   /* nodes per float line of ap_apt1d_run (in registers, with
+                                         three constants per node in shared memory) */
 
 /* Launch shape, chosen by the autotuner (block 0 = library default).  While
  * none is set (no ap_set_launch yet, or the last one with NULL or with every
@@ -465,7 +466,7 @@ int ap_yee1d_run(const ap_yee1d *y, int64_t n_steps, int32_t precision, void *st
  * rounded separately in the stated order (no fused multiply-add); with
  * wp2 = 0 the result is that of ap_yee1d_run bit for bit.  All steps run in
  * one launch, one block per line with the line on chip: float lines of up
- * to 6144 nodes in registers (a few consecutive nodes per thread), longer
+ * to 8192 nodes in registers (two runs of consecutive nodes per thread), longer
  * float lines and double lines in shared memory.
  * Errors: AP_ERR_ARG (nz < 2 or above AP_LINE1D_MAX_NODES_F32/_F64,
  * n_lines < 0, n_steps < 0, NULL arrays, non-finite or non-positive dz, dt,

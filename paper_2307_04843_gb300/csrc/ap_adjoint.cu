@@ -1092,7 +1092,8 @@ __global__ void __launch_bounds__(kAdjBlock, kAdjPairBlocksPerSm)
 // The two-particle kernel's segment length: any split of the steps whose
 // checkpoints (9 floats) and tape (7 floats per step) fit the caller's
 // workspace (n_seg + K states of 12 floats for aa.nslots particles, shared out
-// over `slots` here) gives the same result, and the shorter the segment the
+// over `slots` here) retraces the same states (the gradient's last bits depend on
+// it: each segment is summed in float), and the shorter the segment the
 // smaller the tape.  From 16 steps up it stays in the L2 cache (70 MB of 129 at
 // 16 steps; at 100 steps 436 MB would go through HBM, 56 bytes per
 // particle-step), below 16 the checkpoints' own traffic grows.
@@ -1144,10 +1145,9 @@ int launch_adjoint_k(int precision, const Pulse<double> *dpd, const Pulse<float>
     return gr ? launch_adjoint_t<KIND, AP_FP64, true>(dpd, aa, grid, stream)
               : launch_adjoint_t<KIND, AP_FP64, false>(dpd, aa, grid, stream);
   if (precision == AP_FP32_PHASEFF) {
-    if constexpr (KIND == AP_GAUSS || KIND == AP_FLYING_CF)
-      if (!gr) return launch_adjoint_pair<KIND>(dpf, aa, stream);
-    return gr ? launch_adjoint_t<KIND, AP_FP32_PHASEFF, true>(dpf, aa, grid, stream)
-              : launch_adjoint_t<KIND, AP_FP32_PHASEFF, false>(dpf, aa, grid, stream);
+    if (gr) return launch_adjoint_t<KIND, AP_FP32_PHASEFF, true>(dpf, aa, grid, stream);
+    if constexpr (KIND == AP_GAUSS || KIND == AP_FLYING_CF) return launch_adjoint_pair<KIND>(dpf, aa, stream);
+    else return launch_adjoint_t<KIND, AP_FP32_PHASEFF, false>(dpf, aa, grid, stream);
   }
   return AP_ERR_UNSUPPORTED;
 }

@@ -43,7 +43,7 @@ struct FastPulse {
   float lg_n[6][kLgMaxP];  // the Laguerre recurrences with the subtracted terms' signs in
   float lg_sg, lg_sp, lg_m2w, lg_m4w;  // sgn l, 1 + sgn l (in the frame), -2/w0^2, -4/w0^2
   float r0_hi, r0_lo, rd_hi, rd_lo;    // flying focus: w_first / omega, dw / omega
-  float z_max;            // |Z| beyond which every |zeta_j| > 1e9
+  float z_max;            // |Z| at which the largest |zeta_j| reaches 1e9
   int32_t frame;          // 0: none, 1: x' = y, y' = -x, 2: y' = -y
   int32_t circ;           // circular polarisation
 };
@@ -97,6 +97,10 @@ struct PulseHead {
 template <typename R>
 struct Pulse : PulseHead<R> {
   Comp<R> comp[kMaxComp];
+};
+template <>
+struct Pulse<float> : PulseHead<float> {
+  Comp<float> comp[kMaxComp];
   float4 fcomp[kMaxComp];
 };
 

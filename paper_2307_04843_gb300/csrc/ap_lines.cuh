@@ -52,8 +52,9 @@ struct LineEdge {
 
 // E_0 and B_{nz-1} never change: E_0 belongs to thread 0, and the thread that
 // owns node nz - 1 puts B back after each update (the test is uniform for
-// every other warp).  Nodes past nz - 1 run on zeros and are not stored; they
-// feed nothing but the B that is put back.
+// every other warp).  Nodes past nz - 1 start from zeros, take on whatever the
+// updates give (B_{nz-1} and, on the split line, J1 reach them) and are not
+// stored; they feed nothing but the B that is put back.
 struct LineEnds {
   int ix, iy;      // index of node nz - 1 in this thread's first, second run, or -1
   float keep;      // B_{nz-1}

@@ -456,8 +456,9 @@ struct Turn<F2> {
 // (35 -> 19.5 FP32 operations per component), and its error: the rotation
 // multiplied the rounding of its step by up to n_comp.  Two components share
 // one reciprocal, 1/(d1 d2): 3.5 special-function operations per component.
-// d stays below 2^60 because Z is clamped where every |zeta| reaches 1e9 (the
-// field there is 1e-9 of the focus).
+// d stays below 2^60 because Z is clamped where the largest |zeta| reaches 1e9 (the
+// others follow within the bandwidth's factor; the field there is 1e-9 of the
+// focus).
 template <int POL, typename R>
 __device__ __forceinline__ UnitFields<R> unit_fields_flying(const Pulse<float> &P, const float4 *comps, const float4 st,
                                                             R x, R y, R zhi, R zlo) {
