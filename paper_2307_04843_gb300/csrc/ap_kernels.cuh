@@ -305,17 +305,15 @@ __device__ __forceinline__ double push_d(const Pulse<double> &P, const PushArgs 
 // light-front test, which would otherwise cost every step its branches.
 
 // grid units of the coordinates, and the thread's constants of grid_fetch2:
-// written by the first five threads; the caller synchronises the block before
+// written by the first four threads; the caller synchronises the block before
 // use
 __device__ __forceinline__ void grid_pair_consts(const GridView &g, const StepBase &s, float4 *gk) {
   if (threadIdx.x < 3) {
     const int ax = threadIdx.x;
-    const float f = ax == 2 ? s.gz_s.hi : g.inv_d[ax], o = ax == 2 ? s.gz_o.hi : g.off[ax];
+    const float f = ax == 2 ? s.gz_s : g.inv_d[ax], o = ax == 2 ? s.gz_o.hi : g.off[ax];
     gk[ax] = make_float4(f, f, o, o);
   } else if (threadIdx.x == 3) {
-    gk[3] = make_float4(0.5f, 0.5f, 0.0f, 0.0f);
-  } else if (threadIdx.x == 4) {
-    gk[4] = make_float4(s.gz_s.lo, s.gz_s.lo, s.gz_o.lo, s.gz_o.lo);
+    gk[3] = make_float4(0.5f, 0.5f, s.gz_o.lo, s.gz_o.lo);
   }
 }
 
@@ -328,7 +326,7 @@ struct Caches {
     if constexpr (GRID != kGridNone) grid_slots_init(a, slots);
   }
   __device__ __forceinline__ void fetch(const GridView &g, const StepBase &s, const float4 *, R x, R y, R zhi, R zlo) {
-    const float fz = grid_unit_z(zhi, zlo, s.gz_s.hi, s.gz_o.hi, s.gz_s.lo, s.gz_o.lo);
+    const float fz = grid_unit_z(zhi, zlo, s.gz_s, s.gz_o.hi, s.gz_o.lo);
     grid_fetch_units(g, a, grid_unit<float>(x, g.inv_d[0], g.off[0], g.top[0]),
                      grid_unit<float>(y, g.inv_d[1], g.off[1], g.top[1]), fminf(fmaxf(fz, 0.0f), g.top[2]));
   }
@@ -354,9 +352,8 @@ struct Caches<GRID, F2> {
   }
   __device__ __forceinline__ void fetch(const GridView &g, const StepBase &, const float4 *gk, F2 x, F2 y, F2 zhi,
                                         F2 zlo) {
-    const float4 kz = gk[2], kl = gk[4];
-    grid_fetch2(g, a, b, x, y,
-                grid_unit_z(zhi, zlo, F2(kz.x, kz.y), F2(kz.z, kz.w), F2(kl.x, kl.y), F2(kl.z, kl.w)), gk);
+    const float4 kz = gk[2], kl = gk[3];
+    grid_fetch2(g, a, b, x, y, grid_unit_z(zhi, zlo, F2(kz.x, kz.y), F2(kz.z, kz.w), F2(kl.z, kl.w)), gk);
   }
   __device__ __forceinline__ void values(F2 G[6]) {
     if constexpr (GRID != kGridCellsReg) cp_async_wait_all();
@@ -638,7 +635,7 @@ __device__ __forceinline__ void push_ff_body(const FFPulse<KIND> &P, const StepB
                                              unsigned hist_off) {
   using R = typename std::conditional<NP == 2, F2, float>::type;
   extern __shared__ __align__(16) unsigned char s_dyn[];
-  __shared__ float4 s_gridk[5];
+  __shared__ float4 s_gridk[4];
   __shared__ float4 s_comp[comp_slots<KIND, NP>()];
   if constexpr (KIND == AP_FLYING_SUM) comp_table<R>(P, s_comp);
   if constexpr (NP == 2 && GRID != kGridNone) grid_pair_consts(a.grid, sb, s_gridk);
@@ -747,7 +744,7 @@ __device__ __forceinline__ void batch_body(const Pulse<Real<PREC>> *__restrict__
   PT &sp = *reinterpret_cast<PT *>(s_pulse_raw);
   const PushArgs &a = ba.base;
   const int T = ba.tile;
-  __shared__ float4 s_gridk[5];
+  __shared__ float4 s_gridk[4];
   __shared__ StepBase s_base;
   __shared__ float4 s_comp[kFF ? comp_slots<KIND, NP>() : 1];
   tile_prefix(s_prefix, ba.n_sets, T,

@@ -162,7 +162,8 @@ struct IsPair<F2> : std::true_type {};
 // particle's own warp-uniform refetch branch, as grid_fetch does per particle.
 // fz: the grid unit along z.
 // gk: the factors and offsets from x and y to grid units, pre-broadcast in
-// shared memory, gk[a] = (factor, factor, offset, offset), and gk[3] = (1/2, 1/2, -, -):
+// shared memory, gk[a] = (factor, factor, offset, offset), and gk[3] = (1/2, 1/2, -, -)
+// (-: the low part of the offset along z):
 // a 16-byte load yields both pair operands, where constants kept in the
 // kernel parameters would be re-broadcast into register pairs every step
 // (the two-particle kernels run at their register limit).

@@ -36,7 +36,7 @@
 //   256 Gaussian sets, 4e6 particles x 500 steps     7.43 -> 4.88 ms
 //   CP LG_{1,2}, 3.2e6 x 300                         6.56 -> 4.80 ms
 //   64-component flying focus, 1e6 x 200            15.40 -> 11.52 ms
-//   Gaussian + 256^3 grid, 4e6 x 400                11.62 -> 10.2 ms
+//   Gaussian + 256^3 grid, 4e6 x 400                11.62 -> 10.13 ms
 // The error against 64 bits fell too, to about half (momentum, relative:
 // 1.7e-6 -> 7.6e-7, 1.6e-6 -> 8.9e-7, 7.5e-6 -> 3.3e-7, 1.3e-6 -> 5.8e-7).
 #pragma once
@@ -117,6 +117,14 @@ __host__ __device__ inline double d_add(double a, double b) {
 #endif
 }
 
+__host__ __device__ inline double d_div(double a, double b) {
+#ifdef __CUDA_ARCH__
+  return __ddiv_rn(a, b);
+#else
+  return a / b;
+#endif
+}
+
 struct StepBase {
   FF om0, del;  // carrier phase of step n, in turns: om0 + n del
   FF T0, DT;    // T_n = T0 + n DT: t_n - t_f, for the flying focus in turns of omega
@@ -124,7 +132,8 @@ struct StepBase {
   float h, k;                  // the half and the whole electric kick: -dt/2, -dt
   float hA, hAbr, hAce, hAcb;  // h times the field factors of FastPulse
   float kA, kAce;              // k times them
-  FF gz_s, gz_o;               // grid units along z: Z gz_s + gz_o
+  float gz_s;                  // grid units along z: Z gz_s + gz_o
+  FF gz_o;
 };
 
 __host__ __device__ inline FF d_split(double v) {
@@ -158,21 +167,25 @@ __host__ __device__ inline StepBase make_step_base(const PulseHead<float> &P, do
   s.k = 2.0f * s.h;
   s.kA = 2.0f * s.hA;
   s.kAce = 2.0f * s.hAce;
-  s.gz_s = d_split(d_mul(g.inv_d_d[2], F.z_len));
-  s.gz_o = d_split(d_add(d_mul(P.z_f, g.inv_d_d[2]), g.off_d[2]));
+  // the offset that belongs to the rounded factor: right in the grid's middle, so
+  // within 2^-25 of its half-length at its ends, wherever the focus is
+  const double gs = d_mul(g.inv_d_d[2], F.z_len), mid = d_mul(0.5, (double)(g.nz - 1));
+  s.gz_s = (float)gs;
+  const double o = d_add(d_mul(P.z_f, g.inv_d_d[2]), g.off_d[2]);
+  s.gz_o = d_split(gs != 0.0 ? d_add(mid, -d_mul(d_add(mid, -o), d_div((double)s.gz_s, gs))) : 0.0);
   return s;
 }
 
 // The grid unit of Z = hi + lo.  Z is measured from the focus, so Z s and the
 // offset o cancel when the focus lies away from the grid: their high parts meet
 // in one fused operation, exact up to the rounding of the (small) result, and
-// what that leaves out, the low parts of all three, joins as one correction.
-// The error is then that of the unit itself (2^-24 of it), wherever the focus
-// is; with the high parts alone it grows with the distance (workload 2's grid:
-// 1.5e-5 of a cell with the focus at 0, 3e-3 at 1e4 wavelengths).
+// the low parts join as one correction.  The error is then that of the unit
+// itself (2^-24 of it), wherever the focus is; with the high parts alone it
+// grows with the distance (workload 2's grid: 1.5e-5 of a cell with the focus at
+// 0, 3e-3 at 1e4 wavelengths).
 template <typename R>
-__device__ __forceinline__ R grid_unit_z(R zhi, R zlo, R s_hi, R o_hi, R s_lo, R o_lo) {
-  return radd(rfma(zhi, s_hi, o_hi), rfma(zhi, s_lo, rfma(zlo, s_hi, o_lo)));
+__device__ __forceinline__ R grid_unit_z(R zhi, R zlo, R s, R o_hi, R o_lo) {
+  return radd(rfma(zhi, s, o_hi), rfma(zlo, s, o_lo));
 }
 
 // The step table's entry for step n (an integer below 2^23, in float):
