@@ -37,8 +37,9 @@
 //   CP LG_{1,2}, 3.2e6 x 300                         6.56 -> 4.80 ms
 //   64-component flying focus, 1e6 x 200            15.40 -> 11.52 ms
 //   Gaussian + 256^3 grid, 4e6 x 400                11.62 -> 10.13 ms
-// The error against 64 bits fell too, to about half (momentum, relative:
-// 1.7e-6 -> 7.6e-7, 1.6e-6 -> 8.9e-7, 7.5e-6 -> 3.3e-7, 1.3e-6 -> 5.8e-7).
+// The error against 64 bits fell too, to about half (the largest relative error,
+// norm over norm, of an output, on one set of inputs each: 1.7e-6 -> 7.6e-7, 1.6e-6
+// -> 8.9e-7, 7.5e-6 -> 3.3e-7, 1.3e-6 -> 5.9e-7).
 #pragma once
 
 #include "ap_pair.cuh"
