@@ -1578,17 +1578,24 @@ __global__ void __launch_bounds__(256) nodes_plane_kernel(const __grid_constant_
 }
 
 // Whether plane-wave rows go in runs (see nodes_plane_kernel).  Runs save
-// evaluations, which counts where one is in double or the rows are short; dealt
-// out in turn, neighbouring rows are written at the same time, which counts for
-// wide rows, above all where they end inside a 128-byte line.  Measured, rows in
-// turn / in runs, all components, us: float nodes 250 x 133 x 251 48.8 / 53.4,
-// 1000 x 140 x 140 83.5 / 91.3, 400 x 200 x 200 accumulated 75.6 / 82.4, but
-// 64 x 512 x 300 139 / 96; double nodes 256^3 136 / 130, accumulated 159 /
-// 139, 1000 x 140 x 140 156 / 166, accumulated 160 / 146; evaluated in double
-// 256^3 475 / 138.
+// evaluations, which counts where one is in double or the rows are short, and
+// fill the warps where there are about as many rows as warps; dealt out in turn,
+// neighbouring rows are written at the same time, which counts for many wide
+// rows, above all where they end inside a 128-byte line.  Measured, rows in turn /
+// in runs, all components, us:
+//   float nodes, stored: 250 x 133 x 251 48.8 / 53.4, 1000 x 140 x 140 83.5 / 91.3,
+//     300 x 250 x 200 69.1 / 76.7, but 256 x 136 x 87 (1.2 rows per warp) 33.5 / 32.0,
+//     400 x 136 x 87 37.8 / 33.7, 700 x 136 x 87 again 42.9 / 47.9, 64 x 512 x 300 139 / 96;
+//   float nodes, summed: 400 x 250 x 200 89.2 / 95.8, 288 x 250 x 200 75.1 / 78.5, 250 x 250 x
+//     200 68.8 / 60.2, 700 x 136 x 87 40.1 / 36.4;
+//   double nodes: 256^3 136 / 130, summed 159 / 139, 1000 x 140 x 140 156 / 166, summed
+//     160 / 146; evaluated in double 256^3 475 / 138.
 inline bool plane_runs(int precision, const NodeArgs &a) {
   if (precision != AP_FP32_PHASEFF || a.nx < 192) return true;
-  return a.f64 && (a.accumulate || (a.nx * sizeof(double)) % 128 == 0);
+  const long long rows = (long long)a.ny * a.nz, warps = 64LL * a.sm_count;
+  if (a.f64) return a.accumulate || (a.nx * sizeof(double)) % 128 == 0;
+  if (a.accumulate) return a.nx < 288 || rows < 4 * warps;
+  return a.nx < 640 && rows < 2 * warps;
 }
 
 template <int KIND, int PREC>
