@@ -1477,12 +1477,14 @@ __device__ __forceinline__ void row_put(T *__restrict__ row, int n, W v, bool ac
 // work of 128 columns also where fewer are left; without 16-byte accesses
 // (double nodes, unaligned rows) it stores and sums by single elements, where
 // the row kernel is as wide; and where rows end inside a 32-byte sector, the
-// sectors at the slabs' edges are written in two parts far apart in time.
+// sectors at the slabs' edges are written in two parts far apart in time, which
+// tells once the arrays pass the L2 cache (4e6 nodes are 96 of 129 MB).
 // Measured, slabs / rows, us (1.7e7 nodes where ny allows):
 //   float nodes, stored: nx 256 78 / 93, with ny = 1, 2, 3 97 / 59, 107 / 97, 84 / 96;
 //     nx 64 with ny = 3, 5, 8 67 / 53, 65 / 61, 55 / 61; nx 160 with ny = 3, 4 69 / 65, 61 /
 //     63; unaligned, nx 33 with ny = 6, 12 99 / 84, 100 / 100; rows that end inside a
-//     sector: nx 300 129 / 100, nx 180 138 / 100, nx 250 123 / 108, with ny = 3 99 / 110;
+//     sector: nx 300 129 / 100, nx 180 138 / 100, nx 250 123 / 108, with ny = 3 99 / 110,
+//     in L2: 132 x 95 x 171 23 / 31, 164 x 45 x 97 16.5 / 19.4;
 //   float nodes, summed: nx 256 229 / 397, nx 64 360 / 388, with ny = 1 61 / 44, nx 32
 //     656 / 427; unaligned, nx 250 679 / 400;
 //   double nodes, stored: nx 64 188 / 102, nx 160 156 / 122, nx 250 207 / 191, nx 256
@@ -1492,7 +1494,7 @@ inline bool slab_wins(const NodeArgs &a, bool vec) {
   const bool full = pairs == 2 * slabs;
   if (a.f64) return !a.accumulate && full && a.nx % 4 == 0 && a.ny >= 4;
   if (a.accumulate) return vec && (pairs > slabs || (a.nx == 64 && a.ny > 2));
-  if (slabs > 1 && a.nx % 8 != 0) return full && a.ny >= 3 && a.ny < 6;
+  if (slabs > 1 && a.nx % 8 != 0 && (double)a.nx * a.ny * a.nz >= 4e6) return full && a.ny >= 3 && a.ny < 6;
   if (!vec && pairs == slabs) return a.ny >= 12;
   return (long long)a.ny * pairs >= 6LL * slabs;
 }
